@@ -7,104 +7,172 @@
 // own loop forms X_l = W^T V_l at every l (Alg. 7), which needs twice the
 // recurrence steps.
 //
-// The row range is split into n_split slices; every CTA computes one 64 x 64
-// output tile over one slice and writes its partial sum in float64.  Only the
-// upper tiles of the symmetric G^e are formed.  The partial sums are reduced
-// in a fixed order by moments.cu, so results are bitwise reproducible.
+// The row range is split into n_split slices; every CTA computes one square output tile
+// over one slice and writes its partial sum in float64.  Only elements on or above the
+// diagonal of the symmetric G^e are needed (16 x 16 pieces wholly below it are skipped).
+// The partial sums are reduced in a fixed order by moments.cu, so results are bitwise
+// reproducible.
 #include "internal.h"
 
 namespace ssm {
 
 namespace {
 
-constexpr int TILE = 64;
-constexpr int KT = 32;
+constexpr int KT = 32;  // rows per staged slab
 
-template <typename T, typename Acc>
-__global__ void __launch_bounds__(256)
-gram_kernel(const T* __restrict__ A, const T* __restrict__ B, int ld, int n_tot, int64_t n_rows,
-            int64_t rows_per_split, double* __restrict__ part, int nt1, int n_sym) {
-    __shared__ T Ls[KT][TILE];
-    __shared__ T Rs[KT][TILE];
-    const int tile = blockIdx.x;
-    const int split = blockIdx.y;
-    int which, ti, tj;
-    if (tile < n_sym) {
-        which = 0;
-        // upper-triangular tile index -> (ti, tj), ti <= tj, row-major over ti
-        int r = tile;
-        ti = 0;
-        while (r >= nt1 - ti) {
-            r -= nt1 - ti;
-            ++ti;
-        }
-        tj = ti + r;
-    } else {
+// Tile shapes.  A warp owns one square piece of the tile, 8 x 4 lanes of P x Q outputs,
+// and sums each output over the slice's rows in row order (one fma chain per output), so
+// the shape changes no bit of the result.  Float64 runs at 2 fma a clock and SM here: the
+// kernel is bound by the fma pipe (97 % busy), and what counts is that no warp multiplies
+// padding and that the chains are spread over the SMs.
+//   Wide: 32 x 32 tiles of four 16 x 16 warp pieces.  Pieces past n_tot or below the
+//     diagonal idle.  The Gram pair of two 65536 x 200 float64 blocks: 8.05 ms, 13.7 ms
+//     with 64 x 64 tiles computed whole (1.77 times the useful products; 6.3 ms is the
+//     pipe's floor for these alone).
+//   Mid, Small: one warp a tile, 16 x 16 and 8 x 8, for problems with few tiles and
+//     slices (1024 rows x 40 columns: 545 us in two slices of 64 x 64 tiles, that is on
+//     four SMs).
+// ST: staged slabs (more than two did not help the one-warp tiles: 8.5 against 8.3 ms a
+// call of the 32 x 32 grid, 40 probes, degree 200).
+struct WideTile { static constexpr int P = 2, Q = 4, WR = 2, WC = 2, ST = 2; };
+struct MidTile { static constexpr int P = 2, Q = 4, WR = 1, WC = 1, ST = 2; };
+struct SmallTile { static constexpr int P = 1, Q = 2, WR = 1, WC = 1, ST = 2; };
+
+template <typename S> constexpr int piece() { return 8 * S::P; }
+template <typename S> constexpr int tile_dim() { return piece<S>() * S::WR; }
+
+template <typename T>
+__device__ __forceinline__ void async_elem(T* dst, const T* src, bool ok) {
+    // ok = false: nothing is read and the element is zero
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "n"((int)sizeof(T)), "r"(ok ? (int)sizeof(T) : 0)
+                 : "memory");
+}
+
+// Tile u of the nt1 x nt1 tiles of G^o (which = 1) and the upper ones of G^e, the full
+// tiles before the ragged ones (the light CTAs fill the tail of the launch).
+__device__ __forceinline__ void tile_of_index(int u, int nt1, int n_sym, int& which, int& ti, int& tj) {
+    const int n_all = nt1 * nt1;
+    const bool odd = (int)gridDim.x > n_sym;
+    if (odd && u < n_all) {
         which = 1;
-        const int u = tile - n_sym;
         ti = u / nt1;
         tj = u - ti * nt1;
+        return;
     }
+    which = 0;
+    int r = odd ? u - n_all : u;
+    ti = 0;
+    while (r >= nt1 - ti) {
+        r -= nt1 - ti;
+        ++ti;
+    }
+    tj = ti + r;
+}
+
+template <typename T, typename Acc, typename S>
+__global__ void __launch_bounds__(32 * S::WR * S::WC)
+gram_kernel(const T* __restrict__ A, const T* __restrict__ B, int ld, int n_tot, int64_t n_rows,
+            int64_t rows_per_split, double* __restrict__ part, int nt1, int n_sym) {
+    constexpr int NT = 32 * S::WR * S::WC, TD = tile_dim<S>(), PD = piece<S>(), P = S::P, Q = S::Q;
+    __shared__ __align__(16) T Ls[S::ST][KT][TD];
+    __shared__ __align__(16) T Rs[S::ST][KT][TD];
+    int which, ti, tj;
+    tile_of_index((int)blockIdx.x, nt1, n_sym, which, ti, tj);
     const T* L = A;
-    const T* R = (which == 0) ? A : B;
-    const int64_t r0 = (int64_t)split * rows_per_split;
+    const T* R = which == 0 ? A : B;
+    const int64_t r0 = (int64_t)blockIdx.y * rows_per_split;
     int64_t r1 = r0 + rows_per_split;
     if (r1 > n_rows) r1 = n_rows;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    Acc acc[4][4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int cl0 = ti * TD, cr0 = tj * TD;
+    const int pr = (warp / S::WC) * PD, pc = (warp % S::WC) * PD;  // the warp's piece of the tile
+    const bool on = cl0 + pr < n_tot && cr0 + pc < n_tot && (which == 1 || cr0 + pc + PD > cl0 + pr);
+    const int ri = pr + (lane >> 2) * P, ci = pc + (lane & 3) * Q;
+    Acc acc[P][Q];
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+    for (int p = 0; p < P; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = Acc(0);
-    const int cl0 = ti * TILE, cr0 = tj * TILE;
-    for (int64_t r = r0; r < r1; r += KT) {
-        for (int e = threadIdx.x; e < KT * TILE; e += 256) {
-            const int rr = e / TILE, cc = e - rr * TILE;
+        for (int q = 0; q < Q; ++q) acc[p][q] = Acc(0);
+    auto stage = [&](int buf, int64_t r) {  // rows r .. r + KT - 1 (an empty group past the slice)
+        for (int e = threadIdx.x; e < KT * TD && r < r1; e += NT) {
+            const int rr = e / TD, cc = e - rr * TD;
             const int64_t row = r + rr;
             const bool okr = row < r1;
             const int cl = cl0 + cc, cr = cr0 + cc;
-            Ls[rr][cc] = (okr && cl < n_tot) ? L[row * ld + cl] : T(0);
-            Rs[rr][cc] = (okr && cr < n_tot) ? R[row * ld + cr] : T(0);
+            const bool okl = okr && cl < n_tot, okc = okr && cr < n_tot;
+            async_elem(&Ls[buf][rr][cc], okl ? L + row * ld + cl : L, okl);
+            async_elem(&Rs[buf][rr][cc], okc ? R + row * ld + cr : R, okc);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int q = 0; q + 1 < S::ST; ++q) stage(q, r0 + q * KT);
+    int buf = 0;
+    for (int64_t r = r0; r < r1; r += KT) {
+        stage(buf == 0 ? S::ST - 1 : buf - 1, r + (S::ST - 1) * KT);
+        asm volatile("cp.async.wait_group %0;" ::"n"(S::ST - 1) : "memory");
         __syncthreads();
+        if (on) {
 #pragma unroll 8
-        for (int rr = 0; rr < KT; ++rr) {
-            T a[4], b[4];
+            for (int rr = 0; rr < KT; ++rr) {
+                T a[P], b[Q];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) a[p] = Ls[rr][ty * 4 + p];
+                for (int p = 0; p < P; ++p) a[p] = Ls[buf][rr][ri + p];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) b[q] = Rs[rr][tx * 4 + q];
+                for (int q = 0; q < Q; ++q) b[q] = Rs[buf][rr][ci + q];
 #pragma unroll
-            for (int p = 0; p < 4; ++p)
+                for (int p = 0; p < P; ++p)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[p][q] += Acc(a[p]) * Acc(b[q]);
+                    for (int q = 0; q < Q; ++q) acc[p][q] = fma(Acc(a[p]), Acc(b[q]), acc[p][q]);
+            }
         }
         __syncthreads();
+        if (++buf == S::ST) buf = 0;
     }
-    double* out = part + ((size_t)split * 2 + which) * (size_t)n_tot * n_tot;
+    if (!on) return;
+    double* out = part + ((size_t)blockIdx.y * 2 + which) * (size_t)n_tot * n_tot;
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const int i = cl0 + ty * 4 + p;
+    for (int p = 0; p < P; ++p) {
+        const int i = cl0 + ri + p;
         if (i >= n_tot) continue;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int j = cr0 + tx * 4 + q;
+        for (int q = 0; q < Q; ++q) {
+            const int j = cr0 + ci + q;
             if (j < n_tot) out[(size_t)i * n_tot + j] = (double)acc[p][q];
         }
     }
 }
 
+template <typename T, typename Acc, typename S>
+cudaError_t gram_launch(const T* A, const T* B, int ld, int n_tot, int64_t n_rows, int n_split, int64_t rps,
+                        double* part, cudaStream_t s) {
+    const int nt1 = (n_tot + tile_dim<S>() - 1) / tile_dim<S>();
+    const int n_sym = nt1 * (nt1 + 1) / 2;
+    dim3 grid((unsigned)(n_sym + (B ? nt1 * nt1 : 0)), (unsigned)n_split);
+    gram_kernel<T, Acc, S><<<grid, 32 * S::WR * S::WC, 0, s>>>(A, B, ld, n_tot, n_rows, rps, part, nt1, n_sym);
+    return cudaGetLastError();
+}
+
+template <typename S>
+int64_t gram_ctas(int n_tot, bool odd, int n_split) {
+    const int64_t t = (n_tot + tile_dim<S>() - 1) / tile_dim<S>();
+    return (t * (t + 1) / 2 + (odd ? t * t : 0)) * n_split;
+}
+
+// The widest tile that still gives every SM a CTA (a chain of 512 rows or more per output
+// runs either way; with fewer CTAs than SMs the pipes of the others would idle).
 template <typename T, typename Acc>
 cudaError_t gram(const T* A, const T* B, int ld, int n_tot, int64_t n_rows, int n_split, double* part,
                  cudaStream_t s) {
-    const int nt1 = (n_tot + TILE - 1) / TILE;
-    const int n_sym = nt1 * (nt1 + 1) / 2;
-    const int tiles = n_sym + (B ? nt1 * nt1 : 0);
     int64_t rps = (n_rows + n_split - 1) / n_split;
     rps = (rps + KT - 1) / KT * KT;
-    dim3 grid(tiles, n_split);
-    gram_kernel<T, Acc><<<grid, 256, 0, s>>>(A, B, ld, n_tot, n_rows, rps, part, nt1, n_sym);
-    return cudaGetLastError();
+    const int sms = device_sms();
+    if (gram_ctas<WideTile>(n_tot, B != nullptr, n_split) >= sms)
+        return gram_launch<T, Acc, WideTile>(A, B, ld, n_tot, n_rows, n_split, rps, part, s);
+    if (gram_ctas<MidTile>(n_tot, B != nullptr, n_split) >= sms)
+        return gram_launch<T, Acc, MidTile>(A, B, ld, n_tot, n_rows, n_split, rps, part, s);
+    return gram_launch<T, Acc, SmallTile>(A, B, ld, n_tot, n_rows, n_split, rps, part, s);
 }
 
 __global__ void reduce_gram_pair_kernel(const double* __restrict__ part, int n_split, int n, double* __restrict__ gaa,
@@ -138,7 +206,8 @@ int gram_split_count(int64_t n_rows, int n_tot) {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int nt1 = (n_tot + TILE - 1) / TILE;
+    // slices for about four 64 x 64 tiles an SM (the summation order follows from it)
+    const int nt1 = (n_tot + 63) / 64;
     const int tiles = nt1 * (nt1 + 1) / 2 + nt1 * nt1;
     int64_t want = (4LL * sms + tiles - 1) / tiles;
     int64_t cap = (n_rows + 511) / 512;
