@@ -15,12 +15,12 @@
 // no-swizzle shared-memory operand layout of tcgen05 (K stride 128 B, MN
 // stride 528 B).  This kernel
 // therefore does no conversion: one thread streams panels into a shared-
-// memory ring (stages of the panels' column groups, as many as fit in 133 KB) with
+// memory ring (stages of one to eight panels, as many as fit in 133 KB) with
 // 1-D bulk TMA copies (cp.async.bulk, completion
 // counted in bytes on an mbarrier), one thread issues M=128
 // tcgen05.mma.kind::f16 into TMEM and releases each stage through
 // tcgen05.commit (waiting threads are suspended on the mbarriers, not polling),
-// and at the end all four warps read the accumulators back
+// and at the end all eight warps read the accumulators back
 // with tcgen05.ld and write one float32 partial per slab; partials are
 // reduced in slab order in float64.
 //
@@ -49,7 +49,8 @@ using namespace tc;
 constexpr int KC = 32;                 // rows per panel (K of one pipeline stage)
 constexpr int KG = KC / 8;             // 8-row core groups per panel
 constexpr int STAGES = 16;             // barrier slots (most stages in flight)
-constexpr int NTHREADS = 128;
+constexpr int NTHREADS = 256;
+constexpr int MAX_PS = 8;              // most panels in a stage
 // A column group of a panel is 4 core matrices (512 B) plus a 16-byte pad:
 // with a 528-byte group stride the M/N groups of an MMA operand start on
 // rotating shared-memory banks instead of all on bank 0.
@@ -58,8 +59,16 @@ constexpr int PART_BYTES = 32 * GROUP_BYTES;  // one part of one stage: 32 colum
 constexpr int TMEM_COLS = 512;
 // > half of an SM (one Gram CTA per SM, it owns all 512 TMEM columns) and small enough
 // that two recurrence CTAs (34 KB each) share the SM with it: four one-source stages of
-// 32 column groups.  Stages hold the panels' G groups only, so narrow blocks get more
-// of them in flight (n_tot = 64: 15 one-source or 7 two-source stages).
+// 32 column groups.  Stages hold the panels' G groups only.
+//
+// A stage is PS consecutive panels (one contiguous run of the panel array, one bulk copy
+// a source): as many, up to eight, as leave at least four stages in the ring.  The time
+// of a narrow block is that of the two issuing threads, whose waits, copies and commits
+// come once a stage: with one panel a stage and the tile table in local memory a panel of
+// n_tot = 17 took them ~700 cycles (N = 2.08e6 rows: 478 us, 21 % of the DRAM rate; the
+// KPM line of a 127 x 131 x 125 grid, degree 300: 79.0 ms a call, 46.7 ms with eight).
+// Panels hold ceil(n_tot / 8) groups, not a multiple of two, which takes a quarter off
+// their bytes there.
 constexpr int SMEM_BYTES = 4 * 2 * PART_BYTES + 1024;
 
 struct TcArgs {
@@ -77,7 +86,7 @@ struct TcArgs {
     int both;           // every CTA forms Ge and Go of its slab (n_tot <= 128, PY given)
 };
 
-__global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(TcArgs P) {
+__global__ void __launch_bounds__(NTHREADS, 2) gram_tc_kernel(TcArgs P) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
@@ -98,22 +107,24 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(TcArgs P) {
     const int nch = p1 > p0 ? (int)(p1 - p0) : 0;
     const int nsrc = cross ? 2 : 1;
     const int n_tot = P.n_tot, G = P.G;
-    const int ntp = G * 8;
-    // a stage: nsrc sources x (hi, lo) parts of G groups; an M = 128 operand of the last
-    // part reads up to 16 (G <= 16) or 32 groups from its start, so that much room
-    // follows the ring (rows >= n_tot of the accumulator, never stored)
+    const int ntp = (n_tot + 15) / 16 * 16;  // N of an M = 128 MMA is a multiple of 16
+    // a stage: nsrc sources x PS panels x (hi, lo) parts of G groups.  An M = 128 operand
+    // reads 16 groups and an N operand ntp / 8 from its start: past the part's G groups
+    // that is whatever follows (the next part, the next stage, or the room kept after the
+    // ring), and only accumulator rows and columns >= n_tot, never stored, depend on it.
     const uint32_t part_bytes = (uint32_t)G * GROUP_BYTES;
-    const uint32_t stage_bytes = (uint32_t)nsrc * 2 * part_bytes;
+    const uint32_t panel_bytes = 2 * part_bytes;
     const uint32_t over = (uint32_t)((G <= 16 ? 16 : 32) - G) * GROUP_BYTES;
+    uint32_t PS = 1;
+    while (PS < (uint32_t)MAX_PS && 4u * nsrc * 2 * PS * panel_bytes <= (uint32_t)SMEM_BYTES - over) PS *= 2;
+    const uint32_t src_bytes = PS * panel_bytes;
+    const uint32_t stage_bytes = (uint32_t)nsrc * src_bytes;
     int nstage = (int)((SMEM_BYTES - over) / stage_bytes);
     if (nstage > STAGES) nstage = STAGES;
     if (nstage < 1) nstage = 1;
+    const int nsg = (nch + (int)PS - 1) / (int)PS;  // stages of this slab
     float* out = (cross && !both) ? P.part_o + (size_t)slab * n_tot * n_tot : P.part_e + (size_t)slab * n_tot * n_tot;
 
-    // zero the ring once, so that what an operand reads past the copied groups is 0
-    for (uint32_t t = tid; t < (uint32_t)SMEM_BYTES / 16; t += NTHREADS)
-        reinterpret_cast<uint4*>(smem)[t] = make_uint4(0, 0, 0, 0);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (warp == 0) {
         tmem_alloc(&tmem_slot, TMEM_COLS);
     }
@@ -131,76 +142,81 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(TcArgs P) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_slot;
 
-    // tiles: M block 0 (columns 0..127 of V_{k+1}), M block 1 (128..255)
-    int nt = 1;
-    int t_ag[2] = {0, 16}, t_bg[2] = {0, 0}, t_n[2] = {ntp, 0}, t_dc[2] = {0, ntp}, t_m0[2] = {0, 128},
-        t_n0[2] = {0, 0};
-    bool t_y[2] = {cross, cross};  // B operand from V_k's panels
-    float* t_out[2] = {out, out};
+    // Two tiles at most: M block 0 (columns 0..127 of V_{k+1}) and M block 1 (128..255), or
+    // with `both` Ge and Go of block 0.  A tile's second operand: V_{k+1}'s panels or V_k's
+    // (y), from column group bg, N columns, accumulated in TMEM columns dc ...
+    struct Tile {
+        int ag, bg, n, dc, m0, n0;
+        bool y;
+        float* out;
+    };
+    Tile t0{0, 0, ntp, 0, 0, 0, cross, out}, t1{16, 0, 0, ntp, 128, 0, cross, out};
     if (both) {  // ntp <= 128: tile 0 = Ge, tile 1 = Go in the next ntp columns
-        nt = 2;
-        t_y[0] = false;
-        t_ag[1] = 0;
-        t_n[1] = ntp;
-        t_m0[1] = 0;
-        t_out[1] = P.part_o + (size_t)slab * n_tot * n_tot;
+        t0.y = false;
+        t1 = Tile{0, 0, ntp, ntp, 0, 0, true, P.part_o + (size_t)slab * n_tot * n_tot};
     } else if (ntp > 128) {
-        nt = 2;
         if (!cross) {  // upper blocks only
-            t_bg[1] = 16;
-            t_n[1] = ntp - 128;
-            t_n0[1] = 128;
+            t1.bg = 16;
+            t1.n = ntp - 128;
+            t1.n0 = 128;
         } else {
-            t_n[1] = ntp;
+            t1.n = ntp;
         }
     }
 
     if (warp == 0) {
-        if (lane == 0) {  // producer: bulk copies of panels into the ring
-            const uint32_t copy = (uint32_t)G * GROUP_BYTES;
-            for (int c = 0; c < nch; ++c) {
+        if (lane == 0) {  // producer: bulk copies of runs of panels into the ring
+            const uint8_t* px = P.PX + (size_t)p0 * panel_bytes;
+            const uint8_t* py = P.PY + (size_t)p0 * panel_bytes;
+            for (int c = 0; c < nsg; ++c) {
                 const int s = c % nstage;
                 if (c >= nstage && !mbar_wait_sleep(smem_u32(&empty[s]), ((c / nstage) - 1) & 1, nullptr)) {
                     atomicOr(&fail, 1);
                     break;
                 }
+                const uint32_t np = min(PS, (uint32_t)(nch - c * (int)PS)), bytes = np * panel_bytes;
                 const uint32_t dst = smem_u32(smem + s * stage_bytes);
-                mbar_expect_tx(&full[s], (uint32_t)nsrc * 2 * copy);
-                const int64_t pnl = p0 + c;
-                for (int src = 0; src < nsrc; ++src) {
-                    const uint8_t* base = (src == 0 ? P.PX : P.PY) + (size_t)pnl * 2 * G * GROUP_BYTES;
-                    bulk_copy(dst + (2 * src) * part_bytes, base, copy, &full[s]);
-                    bulk_copy(dst + (2 * src + 1) * part_bytes, base + (size_t)G * GROUP_BYTES, copy, &full[s]);
-                }
+                mbar_expect_tx(&full[s], (uint32_t)nsrc * bytes);
+                bulk_copy(dst, px + (size_t)c * src_bytes, bytes, &full[s]);
+                if (nsrc == 2) bulk_copy(dst + src_bytes, py + (size_t)c * src_bytes, bytes, &full[s]);
             }
         }
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0) {  // MMA issuer
-            const uint32_t lbo = 128, sbo = GROUP_BYTES;
+            // descriptors of the first stage's first panel (the address field counts 16 bytes
+            // and the shared memory ends below 2^18, so offsets are plain additions)
+            const uint64_t base = smem_desc(smem_u32(smem), 128, GROUP_BYTES);
+            const uint32_t part = part_bytes >> 4, panel = panel_bytes >> 4, grp = GROUP_BYTES >> 4;
+            const uint32_t id0 = instr_desc(t0.n), id1 = instr_desc(t1.n);
+            const uint32_t d0 = tmem + (uint32_t)t0.dc, d1 = tmem + (uint32_t)t1.dc;
+            const uint32_t b0 = (t0.y ? src_bytes >> 4 : 0u) + (uint32_t)t0.bg * grp;
+            const uint32_t b1 = (t1.y ? src_bytes >> 4 : 0u) + (uint32_t)t1.bg * grp, a1 = (uint32_t)t1.ag * grp;
+            const bool two = t1.n > 0;
+            uint32_t acc = 0;  // the first MMA into each accumulator overwrites it
             bool ok = true;
-            for (int c = 0; c < nch; ++c) {
+            auto issue = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t id) {
+#pragma unroll
+                for (int kk = 0; kk < KC / 16; ++kk) {
+                    const uint32_t o = 2 * kk * 128 / 16;
+                    mma_bf16(d, a + o, b + o, id, kk == 0 ? acc : 1u);
+                    mma_bf16(d, a + o, b + part + o, id, 1u);
+                    mma_bf16(d, a + part + o, b + o, id, 1u);
+                }
+            };
+            for (int c = 0; c < nsg; ++c) {
                 const int s = c % nstage;
                 if (!mbar_wait_sleep(smem_u32(&full[s]), (c / nstage) & 1, nullptr)) {
                     ok = false;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t xhi = smem_u32(smem + s * stage_bytes), xlo = xhi + part_bytes;
-                for (int t = 0; t < nt; ++t) {
-                    const uint32_t yhi = t_y[t] ? xhi + 2 * part_bytes : xhi;
-                    const uint32_t ylo = t_y[t] ? xhi + 3 * part_bytes : xlo;
-                    const uint32_t idesc = instr_desc(t_n[t]);
-                    const uint32_t dt = tmem + (uint32_t)t_dc[t];
-#pragma unroll
-                    for (int kk = 0; kk < KC / 16; ++kk) {
-                        const uint32_t ao = (uint32_t)t_ag[t] * GROUP_BYTES + 2 * kk * 128;
-                        const uint32_t bo = (uint32_t)t_bg[t] * GROUP_BYTES + 2 * kk * 128;
-                        const uint32_t acc0 = (c == 0 && kk == 0) ? 0u : 1u;
-                        mma_bf16(dt, smem_desc(xhi + ao, lbo, sbo), smem_desc(yhi + bo, lbo, sbo), idesc, acc0);
-                        mma_bf16(dt, smem_desc(xhi + ao, lbo, sbo), smem_desc(ylo + bo, lbo, sbo), idesc, 1u);
-                        mma_bf16(dt, smem_desc(xlo + ao, lbo, sbo), smem_desc(yhi + bo, lbo, sbo), idesc, 1u);
-                    }
+                const uint32_t np = min(PS, (uint32_t)(nch - c * (int)PS));
+                uint64_t x = base + (uint64_t)((uint32_t)s * (stage_bytes >> 4));
+                for (uint32_t p = 0; p < np; ++p, x += panel) {
+                    issue(d0, x, x + b0, id0);
+                    if (two) issue(d1, x + a1, x + b1, id1);
+                    acc = 1;
                 }
                 umma_commit(&empty[s]);
             }
@@ -219,15 +235,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(TcArgs P) {
     if (ok) {
         // each lane holds one accumulator row; 32 columns per TMEM round trip go out
         // through a per-warp 32 x 33 shared-memory tile (the stage ring is free now) as
-        // coalesced 128-byte row stores
+        // coalesced 128-byte row stores; two warps share 32 rows (a warp reaches the TMEM
+        // lanes of its number mod 4) and take every other run of columns
         float* tbuf = reinterpret_cast<float*>(smem) + (size_t)warp * 32 * 33;
-        for (int t = 0; t < nt; ++t) {
-            const int mrow0 = t_m0[t] + 32 * warp;
-            for (int cc = 0; cc < t_n[t]; cc += 32) {
+        auto store = [&](const Tile& t) {
+            const int q = warp & 3, mrow0 = t.m0 + 32 * q;
+            if (mrow0 >= n_tot) return;
+            for (int cc = 32 * (warp >> 2); cc < t.n; cc += 64) {
                 float v[32];
-                const int w = t_n[t] - cc >= 32 ? 32 : 16;
+                const int w = t.n - cc >= 32 ? 32 : 16;
                 if (nch > 0) {
-                    const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(t_dc[t] + cc);
+                    const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(t.dc + cc);
                     if (w == 32)
                         tmem_ld32(ta, v);
                     else
@@ -239,14 +257,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(TcArgs P) {
 #pragma unroll
                 for (int j = 0; j < 32; ++j) tbuf[lane * 33 + j] = v[j];
                 __syncwarp();
-                const int col = t_n0[t] + cc + lane;
-                for (int rr = 0; rr < 32; ++rr) {
-                    const int m = mrow0 + rr;
-                    if (m < n_tot && lane < w && col < n_tot) t_out[t][(size_t)m * n_tot + col] = tbuf[rr * 33 + lane];
+                const int col = t.n0 + cc + lane;
+                if (lane < w && col < n_tot) {
+                    const int nr = min(32, n_tot - mrow0);
+                    for (int rr = 0; rr < nr; ++rr) t.out[(size_t)(mrow0 + rr) * n_tot + col] = tbuf[rr * 33 + lane];
                 }
                 __syncwarp();
             }
-        }
+        };
+        store(t0);
+        if (t1.n > 0) store(t1);
     } else if (tid == 0) {
         atomicOr(P.flag, 2);
     }
@@ -508,7 +528,7 @@ cudaError_t launch_reduce_fused(const float* ring, size_t slot, int nA, int nF, 
 
 bool gram_tc_supported(int n_tot, int ld) { return n_tot >= 1 && n_tot <= 256 && (ld % 4) == 0; }
 
-int gram_tc_groups(int n_tot) { return (n_tot + 15) / 16 * 2; }
+int gram_tc_groups(int n_tot) { return (n_tot + 7) / 8; }
 
 void gram_tc_slabs(int64_t n_rows, int* n_e, int* n_o) {
     int dev = 0, sms = 152;

@@ -246,7 +246,7 @@ bool gram_tc_supported(int n_tot, int ld);
 void gram_tc_slabs(int64_t n_rows, int* n_e, int* n_o);
 size_t gram_tc_partial_floats(int n_e, int n_o, int n_tot);
 size_t gram_tc_partial_floats_total(int n_e, int n_o, int n_tot);  // + room for the float64 sums
-int gram_tc_groups(int n_tot);  // 8-column groups of a panel (n_tot rounded up to 16)
+int gram_tc_groups(int n_tot);  // 8-column groups of a panel
 // both: with a slab table whose Go slabs repeat its Ge slabs (n_o = n_e) and n_tot <= 128,
 // one CTA per slab forms both products (V_{k+1}'s panels read once).
 cudaError_t launch_gram_tc(const uint8_t* PX, const uint8_t* PY, int n_tot, int64_t n_rows, int n_e, int n_o,

@@ -42,8 +42,8 @@ template <typename VT>
 __device__ __forceinline__ VT ldg_stream(const VT* p) { return __ldg(p); }
 
 // Split-bf16 panel of a float32 block for the tensor-core Gram (see
-// gram_tc.cu): rows in panels of 32, columns in groups of 8 (G groups,
-// n_tot rounded up to 16), each (panel, part, group) a 512-byte run of four
+// gram_tc.cu): rows in panels of 32, columns in groups of 8 (G groups; columns past
+// n_tot are zero), each (panel, part, group) a 512-byte run of four
 // 8 x 16-byte core matrices (8 rows x 8 bf16 each) and a 16-byte pad (a
 // 528-byte group stride); part 0 = hi = rn(v),
 // part 1 = lo = rn(v - hi).  The CTA of 8 warps that writes 8 consecutive
