@@ -94,6 +94,9 @@ int64_t batch_points(const Plan& P) {
 }
 constexpr double DECONV_CUTOFF = 1e-14;
 
+// Hybrid columns by the factored routes of the solver (solve.cu): mixed plans.
+bool hybrid_routes(const Plan& P) { return P.mixed && P.p.n_vh > 0; }
+
 ssm_status fail(ssm_plan_s* h, ssm_status st, const std::string& msg) {
     if (h)
         h->P.err = msg;
@@ -377,7 +380,7 @@ ssm_status ensure_points(ssm_plan_s* h, int64_t n_t) {
     }
     if (!h->d_zeta) CUDA_OR_FAIL(h, dev_alloc(&h->d_zeta, M + 1));
     if (!h->d_solve) {
-        CUDA_OR_FAIL(h, dmalloc((void**)&h->d_solve, solve_workspace_bytes(P.p.n_v)));
+        CUDA_OR_FAIL(h, dmalloc((void**)&h->d_solve, solve_workspace_bytes(P.p.n_v, hybrid_routes(P))));
     }
     return SSM_OK;
 }
@@ -526,8 +529,9 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
             // previous such launch, so that the slowest get an SM of their own
             const bool single = t0 == 0 && nb == n_t;
             const int32_t* perm = nullptr;
-            if (single && h->sched_nt == n_t) {
-                const int64_t slots = solve_slots(nv);
+            // (no use where every point runs the serial QL chains)
+            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P))) {
+                const int64_t slots = solve_slots(nv, hybrid_routes(P));
                 if (slots >= n_t) {
                     if ((size_t)slots > h->cap_perm) {
                         dev_free(h->d_perm);
@@ -536,14 +540,15 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
                         CUDA_OR_FAIL(h, dev_alloc(&h->d_perm, (size_t)slots));
                         h->cap_perm = (size_t)slots;
                     }
-                    CUDA_OR_FAIL(h, launch_solve_schedule(h->d_rank, n_t, nv, h->d_perm, P.stream));
+                    CUDA_OR_FAIL(h, launch_solve_schedule(h->d_rank, n_t, nv, hybrid_routes(P), h->d_perm, P.stream));
                     P.stats.launches++;
                     perm = h->d_perm;
                 }
             }
             CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, nv, nvh, P.p.tau, xlo, xhi, muh, M + 1, K,
                                          floor_scale, h->d_solve, h->d_dos_ss + t0, h->d_rank + 2 * t0,
-                                         P.d_flag, P.stream, nullptr, perm, (P.p.options & SSM_OPT_PINV) != 0));
+                                         P.d_flag, P.stream, nullptr, perm, (P.p.options & SSM_OPT_PINV) != 0,
+                                         hybrid_routes(P)));
             P.stats.launches++;
             h->sched_nt = single ? n_t : 0;
         }
@@ -782,7 +787,7 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
                                          P.p.damping ? h->d_muh : h->d_mu, M + 1, K, 0.0,
                                          h->d_solve, h->d_dos_ss + b0 * n_tp, h->d_rank + 2 * b0 * n_tp, P.d_flag,
                                          P.stream, h->d_fpt + 3 * b0 * n_tp, nullptr,
-                                         (P.p.options & SSM_OPT_PINV) != 0));
+                                         (P.p.options & SSM_OPT_PINV) != 0, hybrid_routes(P)));
             P.stats.launches++;
         }
     }
@@ -1952,7 +1957,7 @@ ssm_status ssm_dos_explicit(ssm_plan_t h, const double* W, int64_t ldw, const do
     CUDA_OR_FAIL(h, get(2 * nn, &d_G));
     CUDA_OR_FAIL(h, dmalloc((void**)&d_rank, (size_t)n_t * 2 * sizeof(int32_t)));
     bufs.p.push_back(d_rank);
-    if (!h->d_solve) CUDA_OR_FAIL(h, dmalloc((void**)&h->d_solve, solve_workspace_bytes(nv)));
+    if (!h->d_solve) CUDA_OR_FAIL(h, dmalloc((void**)&h->d_solve, solve_workspace_bytes(nv, false)));
     cudaStream_t st = P.stream;
     CUDA_OR_FAIL(h, cudaMemsetAsync(P.d_flag, 0, sizeof(int), st));
     // W -> V_0 (zero-padded to ld)

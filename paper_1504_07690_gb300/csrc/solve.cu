@@ -23,9 +23,15 @@
 //     and bracketed;
 //   - 0 < r < n in a basis of the kept invariant subspace of K_W (Householder
 //     reduction, Sturm counts, twisted-factorization eigenvectors), then as above;
-//   - otherwise (hybrid columns, a failed check) Alg. 4 step by step: Householder
-//     reduction, accumulated factor, implicit-shift QL (Martin, Reinsch and Wilkinson,
-//     Numer. Math. 11, 1968), bounded at 60 sweeps per eigenvalue.
+//   - otherwise (a failed check; hybrid columns on the float64 plans) Alg. 4 step by step:
+//     Householder reduction, accumulated factor, implicit-shift QL (Martin, Reinsch and
+//     Wilkinson, Numer. Math. 11, 1968), bounded at 60 sweeps per eigenvalue.
+// Hybrid columns on mixed plans take the same routes: C~ spans the kept directions, so
+// ||K_C C~||_F^2 is the squared norm of L^-1 (K_C Y)^T (L L^T = Y^T K_W Y, Y the basis of
+// the kept subspace) on the eigenvectors of the pencil inside the filter (hybrid_norm).
+// The serial QL chains were the time of such points: 400 points of n_v = n_vh = 128 took
+// 94 ms by QL (76 ms unscheduled), 18 ms by the routes.  The float64 plans keep Alg. 4's own steps for them: traces deconvolved with
+// a wide Gaussian weigh these estimates by up to 1e11, so a change of rounding shows.
 // The Householder reduction makes one pass over the lower triangle per column
 // (sym_pass), bisection splits each bracket over a group of lanes, Cholesky factors and
 // AB^T products are blocked through shared-memory tiles.  Matrices live in a per-CTA
@@ -834,7 +840,8 @@ __device__ double trtr_sumsq(const double* __restrict__ L, double* __restrict__ 
 // the tridiagonal's diagonal, in index order) minus theirs.  When more than
 // half of the eigenvalues lie outside, or one of them is far larger than the
 // interval (the subtraction would cancel), the eigenvalues inside are found
-// and summed in index order instead.
+// and summed in index order instead.  sh.misc[2], sh.misc[3]: the index range [jl, jh) of
+// the eigenvalues inside.
 __device__ double range_sum(double* __restrict__ C, int m, double xl, double xh, Shared& sh, int* count) {
     const int tid = threadIdx.x;
     tridiagonalise(C, m, sh);
@@ -860,7 +867,7 @@ __device__ double range_sum(double* __restrict__ C, int m, double xl, double xh,
         if (tid == 0) {
             double tr = 0.0;
             for (int i = 0; i < m; ++i) tr += sh.d[i];
-            int cnt = jhi - jlo;
+            int cnt = jhi - jlo, jl = jlo, jh = jhi;
             double out = 0.0;
             for (int q = 0; q < nout; ++q) out += sh.v[q];
             if (jhi > jlo) {  // edge eigenvalues that rounding puts outside
@@ -868,29 +875,36 @@ __device__ double range_sum(double* __restrict__ C, int m, double xl, double xh,
                 if (!(a0 >= xl && a0 <= xh)) {
                     out += a0;
                     --cnt;
+                    ++jl;
                 }
                 if (jhi - 1 > jlo && !(a1 >= xl && a1 <= xh)) {
                     out += a1;
                     --cnt;
+                    --jh;
                 }
             }
             sh.misc[1] = cnt;
+            sh.misc[2] = jl;
+            sh.misc[3] = jh;
             sh.p[0] = tr - out;
         }
     } else {
         bisect_many(jhi - jlo, [=](int q) { return jlo + q; }, sh.v, m, sh);
         __syncthreads();
         if (tid == 0) {
-            int q = 0;
+            int q = 0, jl = jhi;
             double f = 0.0;
             for (int j = jlo; j < jhi; ++j) {
                 const double xi = sh.v[j - jlo];
                 if (xi >= xl && xi <= xh) {
+                    if (q == 0) jl = j;
                     ++q;
                     f += xi;
                 }
             }
             sh.misc[1] = q;
+            sh.misc[2] = jl;
+            sh.misc[3] = jl + q;
             sh.p[0] = f;
         }
     }
@@ -1314,6 +1328,99 @@ __device__ void reflect_all(double* __restrict__ K1, double* __restrict__ K2, in
     }
 }
 
+// Reflections of Q (column j: the reflector u_j in rows j.., ld ldq, scalar bq[j]) applied
+// in order to the columns of X (m x cols, ld cols): x <- H_{d-1} .. H_0 x.  One column a
+// thread.
+__device__ void reflect_cols(const double* __restrict__ Q, int ldq, const double* __restrict__ bq, int d,
+                             double* __restrict__ X, int m, int cols) {
+    for (int c = threadIdx.x; c < cols; c += (int)blockDim.x)
+        for (int j = 0; j < d; ++j) {
+            const double f =
+                bq[j] * dot8(Q + (size_t)j * ldq + j, ldq, X + (size_t)j * cols + c, cols, m - j);
+#pragma unroll 4
+            for (int i = j; i < m; ++i)
+                X[(size_t)i * cols + c] = fma(-f, Q[(size_t)i * ldq + j], X[(size_t)i * cols + c]);
+        }
+    __syncthreads();
+}
+
+// The basis Y of the kept subspace of K_W: the identity (m = n), the m columns of Q (n x
+// m, ld n), or the trailing m = n - d columns of the d reflections of Q (bq their scalars).
+enum class Basis { Identity, Columns, Reflections };
+
+// The eigenvectors of the pencil in the basis that the range filter keeps: all, or those
+// spanned by the first q columns of H_0 .. H_{q-1} (the reflections of V, ld q, sh.beta),
+// or their complement.
+enum class Kept { All, Span, Complement };
+
+// ||K_C C~||_F^2 of the hybrid correction, K_C = rows nv.. of K (ld n_tot): with L L^T =
+// Y^T K_W Y (L m x m, ld m) the columns of L^-1 (K_C Y)^T hold K_C's coordinates in the
+// K_W-orthonormal basis Y L^-T, and the filter keeps their part in the eigenvectors of the
+// pencil inside it.  The reflections of the eigenvectors' QR split a coordinate vector
+// into the two parts without a subtraction.  The columns go in chunks of at most n through
+// b1, b2 (n^2 each); forward substitution, one column a thread.
+__device__ double hybrid_norm(const double* __restrict__ Kt, int n_tot, int n, int nvh, const double* __restrict__ L,
+                              int m, Basis basis, const double* __restrict__ Q, const double* __restrict__ bq,
+                              Kept kept, const double* __restrict__ V, int q, double* __restrict__ b1,
+                              double* __restrict__ b2, Shared& sh) {
+    const int tid = threadIdx.x, nt = (int)blockDim.x;
+    for (int k = tid; k < m; k += nt) sh.v[k] = 1.0 / L[(size_t)k * m + k];
+    __syncthreads();
+    double f = 0.0;
+    for (int h0 = 0; h0 < nvh; h0 += n) {
+        const int hc = min(n, nvh - h0);
+        for (int e = tid; e < n * hc; e += nt) {
+            const int h = e / n, i = e - h * n;
+            b1[(size_t)i * hc + h] = Kt[(size_t)(n + h0 + h) * n_tot + i];
+        }
+        __syncthreads();
+        double* X = b1;
+        if (basis == Basis::Columns) {
+            gemm_tn(Q, n, b1, hc, n, m, hc, b2, hc, false, sh);
+            X = b2;
+        } else if (basis == Basis::Reflections) {
+            reflect_cols(Q, n, bq, n - m, b1, n, hc);
+            X = b1 + (size_t)(n - m) * hc;
+        }
+        for (int c = tid; c < hc; c += nt)
+            for (int i = 0; i < m; ++i)
+                X[(size_t)i * hc + c] =
+                    (X[(size_t)i * hc + c] - dot8(L + (size_t)i * m, 1, X + c, hc, i)) * sh.v[i];
+        if (kept != Kept::All) {
+            __syncthreads();
+            reflect_cols(V, q, sh.beta, q, X, m, hc);
+        }
+        const int i0 = kept == Kept::Complement ? q : 0, i1 = kept == Kept::Span ? q : m;
+        for (int c = tid; c < hc; c += nt)
+            for (int i = i0; i < i1; ++i) f = fma(X[(size_t)i * hc + c], X[(size_t)i * hc + c], f);
+        __syncthreads();
+    }
+    return block_sum(f, sh.red);
+}
+
+// After range_sum on the m x m matrix C (its reflectors in C, the tridiagonal in sh.d,
+// sh.off, the kept range in sh.misc[2..3]): the reflections of an orthonormal basis of the
+// kept eigenvectors or of the others, whichever are fewer, into V (m x q, ld q; scalars in
+// sh.beta).  Dp, Dm: m x q work.  Returns false if the vectors fail their checks.
+__device__ bool kept_vectors(double* __restrict__ C, int m, double* __restrict__ V, double* __restrict__ Dp,
+                             double* __restrict__ Dm, Kept* kept, int* q_out, Shared& sh) {
+    const int jl = sh.misc[2], jh = sh.misc[3], nin = jh - jl, nout = m - nin;
+    const bool in = nin < nout;
+    const int q = in ? nin : nout;
+    *q_out = q;
+    *kept = in ? Kept::Span : (q ? Kept::Complement : Kept::All);
+    __syncthreads();
+    if (q == 0) return true;
+    bisect_prepare(m, sh);
+    bisect_many(q, [=](int k) { return in ? jl + k : (k < jl ? k : jh + (k - jl)); }, sh.v, m, sh);
+    __syncthreads();
+    twisted_vectors(m, q, V, Dp, Dm, q, sh);
+    if (!sh.misc[6]) return false;
+    back_transform(C, m, V, q, q, sh);
+    householder_qr_cols(V, q, m, q, sh);
+    return true;
+}
+
 // Eigen-decomposition of the symmetric n x n matrix A (destroyed): sh.d gets
 // the eigenvalues; with vectors, row j of Zt the eigenvector of sh.d[j].
 // Without vectors the eigenvalues come from bisection (parallel) instead of
@@ -1338,6 +1445,12 @@ __device__ bool eigh(double* __restrict__ A, double* __restrict__ Zt, int n, boo
     return ql_implicit(Zt, n, vectors, sh);
 }
 
+// Workspace of one CTA in doubles: four n x n buffers; with the routes of hybrid columns
+// (hyb) two more and n scalars.
+__host__ __device__ inline size_t workspace_doubles(int n, bool hyb) {
+    return (size_t)(hyb ? 6 : 4) * n * n + (hyb ? n : 0);
+}
+
 // Trace of an n x n matrix (row-major), the same value on every thread.
 __device__ double diag_sum(const double* M, int n, Shared& sh) {
     double f = 0.0;
@@ -1345,6 +1458,9 @@ __device__ double diag_sum(const double* M, int n, Shared& sh) {
     return block_sum(f, sh.red);
 }
 
+// HYB: hybrid columns take the factored routes (an instance of its own, so that it costs
+// the points without hybrid columns no registers).
+template <bool HYB>
 __global__ void __launch_bounds__(NT, 3)
 solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, int64_t n_t, int nv, int nvh,
              double tau, double xlo, double xhi, const double* __restrict__ mu, int ldmu, int K,
@@ -1369,10 +1485,14 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
     const int tid = threadIdx.x;
     const int n_tot = nv + nvh;
     const size_t nn = (size_t)n * n;
-    double* A = work + (size_t)blockIdx.x * 4 * nn;
+    double* A = work + (size_t)blockIdx.x * workspace_doubles(n, HYB);
     double* Zt = A + nn;
     double* Y = Zt + nn;
     double* T1 = Y + nn;
+    double* U1 = T1 + nn;  // HYB: two more n x n buffers and a vector
+    double* U2 = U1 + nn;
+    double* bq = U2 + nn;
+    const bool routes = HYB || nvh == 0;  // the routes without Alg. 4's eigenvectors
     // slot -> point: the identity, or a schedule that gives the slowest points an SM of
     // their own (perm[slot] < 0: no point)
     for (int64_t sl = blockIdx.x; sl < n_slot; sl += gridDim.x) {
@@ -1393,12 +1513,14 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
             A[e] = 0.5 * (Kt[(size_t)i * n_tot + j] + Kt[(size_t)j * n_tot + i]);
         }
         __syncthreads();
-        // 1'. Without hybrid columns, "every direction is kept" needs no eigenvalues:
+        // 1'. "Every direction is kept" needs no eigenvalues:
         //     g = the largest absolute column sum of K_W bounds smax, and if
         //     K_W - max(tau g, floor) I is positive definite (one Cholesky attempt on T1)
         //     every eigenvalue exceeds max(tau smax, floor), so r = n exactly.
         bool full = false, empty = false;
-        if (nvh == 0) {
+        double kcn = 0.0;       // ||K_C C~||_F^2
+        bool have_kcn = false;
+        if (routes) {
             double g = 0.0;
             for (int j = tid; j < n; j += (int)blockDim.x) {
                 double cs = 0.0;
@@ -1450,7 +1572,7 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
         bool ok = true, done = false;
         if (r_est == 0) {
             done = true;  // K_W(t) is numerically zero: no direction is kept
-        } else if (r_est == n && nvh == 0) {
+        } else if (r_est == n && routes) {
             // 2'. Nothing is truncated, so S~^-1/2 U~^T = S^-1/2 U^T and B = F^-1 K_Z F^-T
             //     with F = U S^1/2 (K_W = F F^T).  For any other factor G = F Q (Q
             //     orthogonal) of K_W, G^-1 K_Z G^-T = Q^T B Q has the same eigenvalues,
@@ -1478,9 +1600,16 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
             }
             __syncthreads();
             if (cholesky_lower(Zt, n, sh)) {
+                r = n;
+                done = true;
                 if (inside) {
                     phi = fma(xl, (double)n, trtr_sumsq(Zt, T1, n, sh));
                     rs = n;
+                    if constexpr (HYB) {
+                        kcn = hybrid_norm(Kt, n_tot, n, nvh, Zt, n, Basis::Identity, nullptr, nullptr, Kept::All,
+                                          nullptr, 0, Y, T1, sh);
+                        have_kcn = true;
+                    }
                 } else {
                     for (int e = tid; e < n * n; e += (int)blockDim.x) {
                         const int i = e / n, j = e - i * n;
@@ -1503,14 +1632,22 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                         rs = n;
                     } else {
                         phi = range_sum(A, n, xl, xh, sh, &rs);
+                        if constexpr (HYB) {
+                            Kept kept;
+                            int q;
+                            have_kcn = kept_vectors(A, n, Y, T1, U1, &kept, &q, sh);
+                            if (have_kcn)
+                                kcn = hybrid_norm(Kt, n_tot, n, nvh, Zt, n, Basis::Identity, nullptr, nullptr, kept,
+                                                  Y, q, U1, U2, sh);
+                            done = have_kcn;
+                        }
                     }
                 }
-                r = n;
-                done = true;
             }
         }
-        bool stale = full;  // A does not hold the tridiagonal form of K_W
-        if (!done && r_est > 0 && r_est < n && nvh == 0) {
+        // A does not hold the tridiagonal form of K_W (the route above got past its factor)
+        bool stale = full || (r_est == n && r == n);
+        if (!done && !full && r_est > 0 && r_est < n && routes) {
             // 2''. Some directions are truncated.  Alg. 4's B is the pencil
             //     (U~^T K_Z U~, U~^T K_W U~ = S~) on the kept invariant subspace of K_W,
             //     and its eigenvalues are the same in any basis Y of that subspace: those
@@ -1521,7 +1658,8 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
             double* Mz = nullptr;  // Y^T K_Z Y
             double* S1 = nullptr;  // free rk x rk buffers for the inertia test
             double* S2 = nullptr;
-            if (3 * dn < rk) {
+            const bool few = 3 * dn < rk;
+            if (few) {
                 // Few dropped directions: Y spans the complement of the dn dropped
                 //     eigenvectors (twisted factorization of the smallest eigenvalues of the
                 //     tridiagonal, back-transformed), as the trailing columns of the
@@ -1541,15 +1679,17 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                     }
                     __syncthreads();
                     reflect_all(Y, T1, n, Zt, n, dn, sh);
+                    Lw = A;
+                    Mz = HYB ? U1 : Zt;  // (K_C's reflections need Zt again)
                     for (int e = tid; e < rk * rk; e += (int)blockDim.x) {  // lower triangles, mirrored
                         const int i = e / rk, j = e - i * rk;
                         const size_t src = (size_t)(dn + max(i, j)) * n + dn + min(i, j);
-                        A[e] = Y[src];
-                        Zt[e] = T1[src];
+                        Lw[e] = Y[src];
+                        Mz[e] = T1[src];
                     }
+                    if (HYB)
+                        for (int j = tid; j < dn; j += (int)blockDim.x) bq[j] = sh.beta[j];
                     __syncthreads();
-                    Lw = A;
-                    Mz = Zt;
                     S1 = Y;
                     S2 = T1;
                     stale = true;
@@ -1578,7 +1718,7 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                     gemm_tn(Zt, n, T1, rk, n, rk, rk, A, rk, true, sh);
                     Lw = Y;
                     Mz = A;
-                    S1 = Zt;
+                    S1 = HYB ? U1 : Zt;  // (K_C Y needs Zt again)
                     S2 = T1;
                     stale = true;
                 }
@@ -1595,9 +1735,17 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                 __syncthreads();
                 const bool inside = !pinv && cholesky_lower(S1, rk, sh) && cholesky_lower(S2, rk, sh);
                 if (cholesky_lower(Lw, rk, sh)) {
+                    [[maybe_unused]] const Basis basis = few ? Basis::Reflections : Basis::Columns;
+                    r = rk;
+                    done = true;
                     if (inside) {
                         phi = fma(xl, (double)rk, trtr_sumsq(Lw, S1, rk, sh));
                         rs = rk;
+                        if constexpr (HYB) {
+                            kcn = hybrid_norm(Kt, n_tot, n, nvh, Lw, rk, basis, Zt, bq, Kept::All, nullptr, 0, T1, U2,
+                                              sh);
+                            have_kcn = true;
+                        }
                     } else {
                         trsm_lower(Lw, Mz, rk, sh);        // Mz = L^-1 M_Z
                         trsm_lower_t(Lw, Mz, T1, rk, sh);  // T1 = L^-1 M_Z L^-T
@@ -1615,14 +1763,22 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                             rs = rk;
                         } else {
                             phi = range_sum(T1, rk, xl, xh, sh, &rs);
+                            if constexpr (HYB) {  // S1, Mz, U2: free (Lw the factor, Zt the basis, T1 reflectors)
+                                Kept kept;
+                                int q;
+                                have_kcn = kept_vectors(T1, rk, S1, Mz, U2, &kept, &q, sh);
+                                if (have_kcn)
+                                    kcn = hybrid_norm(Kt, n_tot, n, nvh, Lw, rk, basis, Zt, bq, kept, S1, q, Mz, U2,
+                                                      sh);
+                                done = have_kcn;
+                            }
                         }
                     }
-                    r = rk;
-                    done = true;
                 }
             }
         }
         if (!done) {
+            rs = 0;
             if (stale) {  // start again from K_W
                 for (int e = tid; e < n * n; e += (int)blockDim.x) {
                     const int i = e / n, j = e - i * n;
@@ -1728,17 +1884,20 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
             }
         }
         if (nvh > 0) {
-            // hybrid correction (Tr K_W~ - ||K_C C~||_F^2) / N~_v; C~ has rs columns (rows of T1)
-            double f = 0.0;
-            for (int e = tid; e < nvh * rs; e += (int)blockDim.x) {
-                const int h = e / rs, mq = e - h * rs;
-                const double* kc = Kt + (size_t)(nv + h) * n_tot;
-                const double* ct = T1 + (size_t)mq * n;
-                double s = 0.0;
-                for (int c = 0; c < n; ++c) s = fma(kc[c], ct[c], s);
-                f = fma(s, s, f);
+            // hybrid correction (Tr K_W~ - ||K_C C~||_F^2) / N~_v; unless the norm is known
+            // already, C~ has rs columns (rows of T1)
+            if (!have_kcn) {
+                double f = 0.0;
+                for (int e = tid; e < nvh * rs; e += (int)blockDim.x) {
+                    const int h = e / rs, mq = e - h * rs;
+                    const double* kc = Kt + (size_t)(nv + h) * n_tot;
+                    const double* ct = T1 + (size_t)mq * n;
+                    double s = 0.0;
+                    for (int c = 0; c < n; ++c) s = fma(kc[c], ct[c], s);
+                    f = fma(s, s, f);
+                }
+                kcn = block_sum(f, sh.red);
             }
-            const double kcn = block_sum(f, sh.red);
             double tr = 0.0;
             for (int h = 0; h < nvh; ++h) tr += Kt[(size_t)(nv + h) * n_tot + nv + h];
             phi += (tr - kcn) / nvh;
@@ -1761,12 +1920,12 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
 int solve_threads(int n_v) { return n_v <= 128 ? 128 : NT; }
 
 // CTAs with a private workspace: 4 x (256 / threads) per SM to overlap the
-// serial QL chains, fewer when 4 n^2 doubles per CTA would exceed 2 GiB in total.
-int workspace_ctas(int n_v) {
+// serial QL chains, fewer when their workspaces would exceed 2 GiB in total.
+int workspace_ctas(int n_v, bool hyb) {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const size_t per = (size_t)4 * n_v * n_v * sizeof(double);
+    const size_t per = workspace_doubles(n_v, hyb) * sizeof(double);
     size_t cap = ((size_t)2 << 30) / per;
     size_t g = (size_t)4 * sms * (NT / solve_threads(n_v));
     if (g > cap) g = cap;
@@ -1779,8 +1938,8 @@ size_t solve_smem(int n) {
 
 }  // namespace
 
-size_t solve_workspace_bytes(int n_v) {
-    return (size_t)workspace_ctas(n_v) * 4 * (size_t)n_v * n_v * sizeof(double);
+size_t solve_workspace_bytes(int n_v, bool hyb) {
+    return (size_t)workspace_ctas(n_v, hyb) * workspace_doubles(n_v, hyb) * sizeof(double);
 }
 
 // Schedule of the next solve launch from the routes of the previous one (its kept
@@ -1839,41 +1998,44 @@ __global__ void solve_schedule_kernel(const int32_t* __restrict__ rank_prev, int
 cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int n_v, int n_vh, double tau,
                          double xlo, double xhi, const double* mu, int ldmu, int K, double floor_scale, void* work,
                          double* dos, int32_t* rank, int* flag, cudaStream_t s, const double* floor_pt,
-                         const int32_t* perm, bool pinv) {
+                         const int32_t* perm, bool pinv, bool hyb) {
     if (n_t <= 0) return cudaSuccess;
     if (n_v > MAXN) return cudaErrorInvalidValue;
     const size_t smem = solve_smem(n_v);
-    cudaError_t e = cudaFuncSetAttribute(solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kernel = hyb ? solve_kernel<true> : solve_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    int64_t grid = workspace_ctas(n_v), n_slot = n_t;
+    int64_t grid = workspace_ctas(n_v, hyb), n_slot = n_t;
     if (perm) {
-        n_slot = solve_slots(n_v);
+        n_slot = solve_slots(n_v, hyb);
         if (n_slot < n_t || n_slot > grid) return cudaErrorInvalidValue;
     }
     if (grid > n_slot) grid = n_slot;
-    solve_kernel<<<(int)grid, solve_threads(n_v), smem, s>>>(Kfull, KZ, n_t, n_v, n_vh, tau, xlo, xhi, mu, ldmu, K,
+    kernel<<<(int)grid, solve_threads(n_v), smem, s>>>(Kfull, KZ, n_t, n_v, n_vh, tau, xlo, xhi, mu, ldmu, K,
                                                    floor_scale, (double*)work, dos, rank, flag, floor_pt, perm,
                                                    n_slot, pinv);
     return cudaGetLastError();
 }
 
-int64_t solve_slots(int n_v) {
+int64_t solve_slots(int n_v, bool hyb) {
     int dev = 0, sms = 0, k = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = solve_smem(n_v);
-    if (cudaFuncSetAttribute(solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, solve_kernel, solve_threads(n_v), smem) != cudaSuccess)
+    const auto kernel = hyb ? solve_kernel<true> : solve_kernel<false>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, kernel, solve_threads(n_v), smem) != cudaSuccess)
         return 0;
     const int64_t slots = (int64_t)sms * k;
-    return slots <= workspace_ctas(n_v) ? slots : 0;
+    return slots <= workspace_ctas(n_v, hyb) ? slots : 0;
 }
 
-cudaError_t launch_solve_schedule(const int32_t* rank_prev, int64_t n_t, int n_v, int32_t* perm, cudaStream_t s) {
+cudaError_t launch_solve_schedule(const int32_t* rank_prev, int64_t n_t, int n_v, bool hyb, int32_t* perm,
+                                  cudaStream_t s) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t slots = solve_slots(n_v);
+    const int64_t slots = solve_slots(n_v, hyb);
     if (slots < n_t || slots <= 0) return cudaErrorInvalidValue;
     const size_t smem = (size_t)(slots + n_t) * sizeof(int32_t);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
