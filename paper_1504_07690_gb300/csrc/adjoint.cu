@@ -21,13 +21,14 @@
 // per-axis coupling: sum over edges of <U_{k+1}[i], V_k[j]> regrouped by the
 // symmetric neighbour relation), or for CSR <U_{k+1}[i], V_k[j]> per stored
 // entry.  Each row's terms are summed across lanes in a fixed shuffle tree
-// and added to per-row (per-entry) float64 accumulators, so results do not
-// depend on scheduling.  When every G_l is a multiple of the identity (the
+// and added to per-row (per-entry) float64 accumulators, one addition per element and
+// launch, so results do not depend on scheduling.  When every G_l is a multiple of the identity (the
 // losses of Alg. 2's KPM line and of Tr f(A)) Gbar_k is three scaled blocks,
 // fused into the step; general G_l go through a tiled GEMM first.
 #include <type_traits>
 
 #include "internal.h"
+#include "sweep.cuh"
 
 namespace ssm {
 
@@ -62,23 +63,49 @@ struct AdjScalars {
     double gcoef;        // weight of the pair (U_{k+1}, V_k) in dL/dA~ (0: no gradient terms)
 };
 
+// One value of four (selected by the lane) summed over the W lanes of a row, W = 4 .. 32:
+// v[0..3] of every lane are added over the lane offsets W/2, W/4, .. 1 in that order, as a
+// shuffle tree of each value would, but the first two offsets also halve the values a lane
+// carries (6 shuffles instead of 20 at W = 32).  Returns v[4 (lane mod W) / W] summed;
+// lanes 0, W/4, W/2 and 3W/4 of a row hold the four.
+template <int W, typename T>
+__device__ __forceinline__ T row_sum4(const T* v, uint32_t lane) {
+    const bool up = lane & (W / 2), up2 = lane & (W / 4);
+    T a = up ? v[2] : v[0], b = up ? v[3] : v[1];
+    a += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], W / 2);
+    b += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], W / 2);
+    T c = up2 ? b : a;
+    c += __shfl_xor_sync(0xffffffffu, up2 ? a : b, W / 4);
+#pragma unroll
+    for (int o = W / 8; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    return c;
+}
+
 // Stencil step.  Un1 = U_{k+1}, Un2 = U_{k+2}, Vm/V0/Vp = V_{k-1}, V_k, V_{k+1}; Gb
 // (nullable) a precomputed Gbar_k; Uo (nullable) receives U_k.  D[i] and E[3 i + d]
 // accumulate gcoef <U_{k+1}[i], V_k[i]> and gcoef <V_k[i], nbr_d(U_{k+1})[i]>.
-template <typename T>
+// W lanes share a row (the power of two >= nchunk, at most 32; a row of a narrow block
+// fills a quarter of a warp, not one).  The accumulators take one fire-and-forget addition
+// each (one per element and launch, so their order is that of the launches): a load, an
+// add and a store there, after the tree of 20 shuffles, held every warp for a second
+// memory latency per row (10^6 rows of 128 columns: 1.40 ms,
+// 1.14 without it).
+template <typename T, int W>
 __global__ void __launch_bounds__(256)
 adj_stencil_kernel(const T* __restrict__ Un1, const T* __restrict__ Un2, const T* __restrict__ Vm,
                    const T* __restrict__ V0, const T* __restrict__ Vp, const T* __restrict__ Gb, T* __restrict__ Uo,
                    const T* __restrict__ diag2, StencilGeom g, T o0, T o1, T o2, AdjScalars sc,
                    double* __restrict__ D, double* __restrict__ E, uint32_t nchunk, uint32_t n_rows) {
     using VT = typename V16<T>::type;
-    const uint32_t lane = threadIdx.x & 31;
+    constexpr uint32_t RW = 32 / W;  // rows a warp
+    const uint32_t lane = threadIdx.x & 31, wl = lane & (W - 1), sub = lane / W;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     const T w[3] = {g.active[0] ? o0 : T(0), g.active[1] ? o1 : T(0), g.active[2] ? o2 : T(0)};
     const uint32_t ext[3] = {g.d0, g.d1, g.d2};
     const uint32_t sd[3] = {g.d1 * g.d2, g.d2, 1u};
     const T ga = (T)sc.ga, gb = (T)sc.gb, gc = (T)sc.gc;
     const bool grad = sc.gcoef != 0.0;
+    const bool has_a = Uo && !Gb && ga != T(0), has_b = gb != T(0), has_c = Uo && !Gb && gc != T(0);
     const VT* un1 = reinterpret_cast<const VT*>(Un1);
     const VT* un2 = reinterpret_cast<const VT*>(Un2);
     const VT* vm = reinterpret_cast<const VT*>(Vm);
@@ -86,7 +113,10 @@ adj_stencil_kernel(const T* __restrict__ Un1, const T* __restrict__ Un2, const T
     const VT* vp = reinterpret_cast<const VT*>(Vp);
     const VT* gbar = reinterpret_cast<const VT*>(Gb);
     VT* uo = reinterpret_cast<VT*>(Uo);
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n_rows; i += warps) {
+    const uint64_t step = (uint64_t)warps * RW;
+    for (uint64_t i0 = (uint64_t)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * RW; i0 < n_rows; i0 += step) {
+        const uint32_t i = (uint32_t)i0 + sub;
+        const bool live = i < n_rows;
         const uint32_t c2 = i % g.d2, q = i / g.d2, c1 = q % g.d1, c0 = q / g.d1;
         const uint32_t co[3] = {c0, c1, c2};
         uint32_t nb[6];
@@ -102,46 +132,186 @@ adj_stencil_kernel(const T* __restrict__ Un1, const T* __restrict__ Un2, const T
             nb[2 * a + 1] = cm + 1 < e ? i + st : i - (e - 1) * st;
         }
         const size_t base = (size_t)i * nchunk;
-        const T d2 = diag2[i];
-        T dd = T(0), de[3] = {T(0), T(0), T(0)};
-        for (uint32_t cc = lane; cc < nchunk; cc += 32) {
+        T dt[4] = {T(0), T(0), T(0), T(0)};  // dd, de[0..2]
+        for (uint32_t cc = wl; live && cc < nchunk; cc += W) {
+            // every load before the first use
             const VT x = un1[base + cc];
             const VT vk = v0[base + cc];
-            VT acc = axpyv(d2, x, zerov(T(0)));
+            VT nv[6];
+#pragma unroll
+            for (int a = 0; a < 6; ++a)
+                nv[a] = (has >> a) & 1u ? un1[(size_t)nb[a] * nchunk + cc] : zerov(T(0));
+            const VT u2 = uo ? un2[base + cc] : zerov(T(0));
+            const VT gv = (uo && gbar) ? gbar[base + cc] : (has_a ? vm[base + cc] : zerov(T(0)));
+            const VT vc = has_c ? vp[base + cc] : zerov(T(0));
+            VT acc = axpyv(diag2[i], x, zerov(T(0)));
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const bool lo = (has >> (2 * a)) & 1u, hi = (has >> (2 * a + 1)) & 1u;
                 if (lo || hi) {
                     VT s = zerov(T(0));
-                    if (lo) s = addv(s, un1[(size_t)nb[2 * a] * nchunk + cc]);
-                    if (hi) s = addv(s, un1[(size_t)nb[2 * a + 1] * nchunk + cc]);
+                    if (lo) s = addv(s, nv[2 * a]);
+                    if (hi) s = addv(s, nv[2 * a + 1]);
                     acc = axpyv(w[a], s, acc);
-                    if (grad) de[a] += dotv(vk, s);
+                    if (grad) dt[a + 1] += dotv(vk, s);
                 }
             }
-            if (grad) dd += dotv(x, vk);
+            if (grad) dt[0] += dotv(x, vk);
             if (uo) {
-                VT out = subv(acc, un2[base + cc]);
+                VT out = subv(acc, u2);
                 if (gbar) {
-                    out = addv(out, gbar[base + cc]);
+                    out = addv(out, gv);
                 } else {
-                    if (ga != T(0)) out = axpyv(ga, vm[base + cc], out);
-                    if (gb != T(0)) out = axpyv(gb, vk, out);
-                    if (gc != T(0)) out = axpyv(gc, vp[base + cc], out);
+                    if (has_a) out = axpyv(ga, gv, out);
+                    if (has_b) out = axpyv(gb, vk, out);
+                    if (has_c) out = axpyv(gc, vc, out);
                 }
                 uo[base + cc] = out;
             }
         }
         if (grad) {
-            dd = warp_sum(dd);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) de[a] = warp_sum(de[a]);
-            if (lane == 0) {
-                D[i] += sc.gcoef * (double)dd;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) E[3 * (size_t)i + a] += sc.gcoef * (double)de[a];
+            const T sum = row_sum4<W>(dt, lane);
+            if (live && (wl & (W / 4 - 1)) == 0) {
+                const uint32_t v = wl / (W / 4);
+                atomicAdd(v == 0 ? D + i : E + 3 * (size_t)i + (v - 1), sc.gcoef * (double)sum);
             }
         }
+    }
+}
+
+// The stencil step of adj_stencil_kernel by sweeps (sweep.cuh) for rows of at most W chunks:
+// 512 threads own a tile of 512 / W whole rows (so the row sums stay inside a warp), and
+// the tile's U_{k+1} with its halo, U_{k+2} and the V blocks stream through the ring, three
+// planes ahead.  The row-at-a-time kernel re-reads U_{k+1} from L2 for each of its seven
+// uses and leaves each warp one memory latency a row with 46 % of the copy rate (1.14 ms at
+// 10^6 rows of 128 columns; 0.70 ms here, 0.65 of the copy rate); here ~150 KB a SM are in
+// flight all the time.  Same operations
+// in the same order; what an open edge lacks is a zero in the ring.
+template <int W> struct AdjTile;
+template <> struct AdjTile<32> { using T = SweepTile<4, 4, 3>; };
+template <> struct AdjTile<16> { using T = SweepTile<4, 8, 3>; };
+template <> struct AdjTile<8> { using T = SweepTile<8, 8, 3>; };
+template <> struct AdjTile<4> { using T = SweepTile<8, 16, 3>; };
+
+template <int W>
+constexpr size_t adj_sweep_smem() {
+    using ST = typename AdjTile<W>::T;
+    return (size_t)ST::NSLOT * (ST::PLANE + 4 * ST::ROWS) * W * 16;
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(512)
+adj_sweep_kernel(const T* __restrict__ Un1, const T* __restrict__ Un2, const T* __restrict__ Vm,
+                 const T* __restrict__ V0, const T* __restrict__ Vp, const T* __restrict__ Gb, T* __restrict__ Uo,
+                 const T* __restrict__ diag2, StencilGeom g, T o0, T o1, T o2, AdjScalars sc, double* __restrict__ D,
+                 double* __restrict__ E, uint32_t nchunk, uint32_t nt2, uint32_t planes) {
+    using VT = typename V16<T>::type;
+    using ST = typename AdjTile<W>::T;
+    constexpr uint32_t PL = ST::PLANE * W, RW = ST::ROWS * W, SLOT = PL + 4 * RW;
+    extern __shared__ __align__(16) uint8_t adj_smem[];
+    VT* ring = reinterpret_cast<VT*>(adj_smem);  // NSLOT x (plane of U_{k+1}; U_{k+2}, V_k, Gbar or V_{k-1}, V_{k+1})
+    const int d0 = (int)g.d0, d1 = (int)g.d1, d2 = (int)g.d2;
+    const uint32_t cc = threadIdx.x % W, lane = threadIdx.x & 31;
+    const SweepRow<ST> R((int)(threadIdx.x / W));
+    const int b1 = (int)(blockIdx.x / nt2) * ST::T1, b2 = (int)(blockIdx.x % nt2) * ST::T2;
+    const int z0 = (int)(blockIdx.y * planes), z1 = min(z0 + (int)planes, d0);
+    const bool col = cc < nchunk, per0 = g.per[0] != 0;
+    const T w0 = g.active[0] ? o0 : T(0), w1 = g.active[1] ? o1 : T(0), w2 = g.active[2] ? o2 : T(0);
+    const T ga = (T)sc.ga, gb = (T)sc.gb, gc = (T)sc.gc;
+    const bool grad = sc.gcoef != 0.0, write = Uo != nullptr;
+    const bool has_g = write && Gb, has_a = write && !Gb && ga != T(0), has_b = gb != T(0),
+               has_c = write && !Gb && gc != T(0);
+    // neighbours along an axis of extent 1 are the row itself (folded into the diagonal)
+    const bool on1 = d1 > 1, on2 = d2 > 1;
+    const int p1 = b1 + R.r1, p2 = b2 + R.r2;
+    const int m1 = axis_at(p1, d1, g.per[1] && on1), m2 = axis_at(p2, d2, g.per[2] && on2);
+    const bool own = col && m1 >= 0 && m2 >= 0;
+    const bool live = p1 < d1 && p2 < d2, out_row = col && live;
+    const int q1 = axis_at(b1 + R.h1, d1, g.per[1] && on1), q2 = axis_at(b2 + R.h2, d2, g.per[2] && on2);
+    const bool hok = R.halo && col && q1 >= 0 && q2 >= 0 && (R.ax1 ? on1 : on2);
+    const size_t pstride = (size_t)d1 * d2 * nchunk;
+    const VT* un1 = reinterpret_cast<const VT*>(Un1);
+    const size_t eown = own ? ((size_t)m1 * d2 + m2) * nchunk + cc : 0;
+    const size_t ehal = hok ? ((size_t)q1 * d2 + q2) * nchunk + cc : 0;
+    const uint32_t so = R.own_at() * W + cc, sh = R.halo_at() * W + cc, st = PL + threadIdx.x;
+    const VT zero = zerov(T(0));
+    const size_t orow = live ? (size_t)p1 * d2 + p2 : 0, eout = orow * nchunk + cc;
+    const uint32_t prow = (uint32_t)(d1 * d2);
+    const VT* third = reinterpret_cast<const VT*>(has_g ? Gb : Vm);
+    auto stage = [&](int z, uint32_t slot) {
+        if (z <= z1) {
+            const int m = axis_at(z, d0, per0);
+            const size_t off = (size_t)(m < 0 ? 0 : m) * pstride;
+            VT* S = ring + slot * SLOT;
+            async16(S + so, un1 + off + eown, own && m >= 0);
+            if (z >= z0 && z < z1) {
+                if (R.halo) async16(S + sh, un1 + off + ehal, hok);
+                if (out_row) {
+                    if (write) async16(S + st, reinterpret_cast<const VT*>(Un2) + off + eout, true);
+                    async16(S + st + RW, reinterpret_cast<const VT*>(V0) + off + eout, true);
+                    if (has_g || has_a) async16(S + st + 2 * RW, third + off + eout, true);
+                    if (has_c) async16(S + st + 3 * RW, reinterpret_cast<const VT*>(Vp) + off + eout, true);
+                }
+            }
+        }
+        async_commit();
+    };
+#pragma unroll
+    for (int q = 0; q < ST::NSLOT; ++q) stage(z0 - 1 + q, q);
+    T dg = out_row ? diag2[(size_t)z0 * prow + orow] : T(0);
+    async_wait<ST::PF - 1>();  // planes z0 - 1, z0
+    VT xm = ring[so], xc = ring[SLOT + so];
+    uint32_t slot = 1;  // of plane z
+    for (int z = z0; z < z1; ++z) {
+        async_wait<ST::PF - 2>();  // planes up to z + 1
+        __syncthreads();           // ... of every thread; and plane z - 1 is read by none any more
+        stage(z + ST::PF, slot == 0 ? ST::NSLOT - 1 : slot - 1);
+        const VT* S = ring + slot * SLOT;
+        const uint32_t next = slot + 1 == ST::NSLOT ? 0 : slot + 1;
+        const VT xp = ring[next * SLOT + so];
+        const T dgn = out_row && z + 1 < z1 ? diag2[(size_t)(z + 1) * prow + orow] : T(0);
+        T dt[4] = {T(0), T(0), T(0), T(0)};  // <U_{k+1}, V_k>, then per axis
+        if (out_row) {
+            const VT vk = S[st + RW];
+            const VT s0 = addv(addv(zero, xm), xp);
+            VT acc = axpyv(dg, xc, zero);
+            acc = axpyv(w0, s0, acc);
+            if (grad) dt[1] = dotv(vk, s0);
+            if (on1) {
+                const VT s1 = addv(addv(zero, S[so - ST::W2 * W]), S[so + ST::W2 * W]);
+                acc = axpyv(w1, s1, acc);
+                if (grad) dt[2] = dotv(vk, s1);
+            }
+            if (on2) {
+                const VT s2 = addv(addv(zero, S[so - W]), S[so + W]);
+                acc = axpyv(w2, s2, acc);
+                if (grad) dt[3] = dotv(vk, s2);
+            }
+            if (grad) dt[0] = dotv(xc, vk);
+            if (write) {
+                VT out = subv(acc, S[st]);
+                if (has_g) {
+                    out = addv(out, S[st + 2 * RW]);
+                } else {
+                    if (has_a) out = axpyv(ga, S[st + 2 * RW], out);
+                    if (has_b) out = axpyv(gb, vk, out);
+                    if (has_c) out = axpyv(gc, S[st + 3 * RW], out);
+                }
+                reinterpret_cast<VT*>(Uo)[(size_t)z * pstride + eout] = out;
+            }
+        }
+        if (grad) {
+            const T sum = row_sum4<W>(dt, lane);
+            if (live && (cc & (W / 4 - 1)) == 0) {
+                const uint32_t v = cc / (W / 4);
+                const size_t i = (size_t)z * prow + orow;
+                atomicAdd(v == 0 ? D + i : E + 3 * i + (v - 1), sc.gcoef * (double)sum);
+            }
+        }
+        xm = xc;
+        xc = xp;
+        dg = dgn;
+        slot = next;
     }
 }
 
@@ -381,8 +551,32 @@ static cudaError_t adj_step(const Plan& P, const T* Un1, const T* Un2, const T* 
         const T o0 = std::is_same<T, float>::value ? (T)P.off32[0] : (T)P.off64[0];
         const T o1 = std::is_same<T, float>::value ? (T)P.off32[1] : (T)P.off64[1];
         const T o2 = std::is_same<T, float>::value ? (T)P.off32[2] : (T)P.off64[2];
-        adj_stencil_kernel<T><<<rows_grid(P.n), 256, 0, s>>>(Un1, Un2, Vm, V0, Vp, Gb, Uo, diag2, P.geom, o0, o1,
-                                                             o2, sc, D, EF, nchunk, (uint32_t)P.n);
+        auto run = [&](auto width) -> cudaError_t {
+            constexpr int W = decltype(width)::value;
+            using ST = typename AdjTile<W>::T;
+            // one 512-thread CTA an SM (its ring): about eight CTAs an SM over the launch.
+            // Below 12 MiB a block the L2 feeds the row-at-a-time kernel and a run's planes
+            // are a serial chain (100 steps: 1.9 against 3.1 ms at 4 MiB, 2.6 against 3.9
+            // at 5, 6.0 against 4.1 at 17, 18 against 12 at 57).
+            const SweepRuns w =
+                sweep_runs<ST>(P.geom.d0, P.geom.d1, P.geom.d2, 1, (uint64_t)device_sms() * 8, 16);
+            if (w.nseg && nchunk <= W && (uint64_t)P.n * nchunk * 16 >= (12ull << 20)) {
+                constexpr size_t smem = adj_sweep_smem<W>();
+                const cudaError_t e = cudaFuncSetAttribute(adj_sweep_kernel<T, W>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+                adj_sweep_kernel<T, W><<<dim3(w.nt1 * w.nt2, w.nseg), 512, smem, s>>>(
+                    Un1, Un2, Vm, V0, Vp, Gb, Uo, diag2, P.geom, o0, o1, o2, sc, D, EF, nchunk, w.nt2, w.planes);
+            } else {
+                adj_stencil_kernel<T, W><<<rows_grid((P.n * W + 31) / 32), 256, 0, s>>>(
+                    Un1, Un2, Vm, V0, Vp, Gb, Uo, diag2, P.geom, o0, o1, o2, sc, D, EF, nchunk, (uint32_t)P.n);
+            }
+            return cudaGetLastError();
+        };
+        if (nchunk <= 4) return run(std::integral_constant<int, 4>{});
+        if (nchunk <= 8) return run(std::integral_constant<int, 8>{});
+        if (nchunk <= 16) return run(std::integral_constant<int, 16>{});
+        return run(std::integral_constant<int, 32>{});
     } else {
         const T* val2 = std::is_same<T, float>::value ? (const T*)P.d_val32 : (const T*)P.d_val64;
         adj_csr_kernel<T><<<rows_grid(P.n), 256, 0, s>>>(Un1, Un2, Vm, V0, Vp, Gb, Uo, P.d_rowptr, P.d_colind, val2,
