@@ -16,6 +16,7 @@
 
 
 #include "internal.h"
+#include "sweep.cuh"
 
 namespace ssm {
 
@@ -339,6 +340,114 @@ stencil_march_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp,
     }
 }
 
+// Float32 stencil step on large 3D grids, by sweeps: a CTA owns an 8 x 8 tile of axes 1
+// and 2 and C 16-byte column chunks, and sweeps a run of planes along axis 0.  A thread
+// keeps its element of planes z - 1, z, z + 1 in registers; the plane's tile and its halo of
+// 32 rows go through shared memory, so an element of V_k is read 1.5 times instead of once
+// per neighbour, and the loads of plane z + 2, of the next halo and of V_{k-1} are in
+// flight while plane z is computed.  Neighbours past an open edge are zeros in shared
+// memory, which the sums pass unchanged; the operations and their order are those of
+// stencil_step_kernel, so the outputs are the same values (a zero may change sign).
+// What bounds it: memory.  On a 100^3 grid of 128 columns without panels 308 us and 3.6 GB
+// between L2 and the SMs, against 328 us and 5.0 GB for the per-item kernel; with panels
+// beside the Gram products a 64^3 grid of 256 columns takes 0.34 ms a step instead of 0.36.
+// (A ring of asynchronous copies instead of the registers was slower there, 0.35 ms: the
+// Gram CTA holds most of the shared memory; so were sweeps along axis 1 of 2D grids, 68-76
+// ms a call against 61.6 ms on the 256^2 one.)
+using Tile3D = SweepTile<8, 8, 1>;
+
+template <bool PANEL>
+__global__ void __launch_bounds__(512)
+stencil_sweep_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp, float* __restrict__ Vn,
+                     const float* __restrict__ diag2, StencilGeom g, float o0, float o1, float o2, float c, float d,
+                     uint32_t nchunk, uint32_t C, uint32_t ngrp, uint32_t nt2, uint32_t planes, PanelOut po) {
+    using ST = Tile3D;
+    extern __shared__ __align__(16) float4 sw[];  // two staged planes
+    const int d0 = (int)g.d0, d1 = (int)g.d1, d2 = (int)g.d2;
+    const uint32_t grp = blockIdx.x % ngrp, tile = blockIdx.x / ngrp;
+    const int b1 = (int)(tile / nt2) * ST::T1, b2 = (int)(tile % nt2) * ST::T2;
+    const uint32_t cl = threadIdx.x % C, cc = grp * C + cl;
+    const SweepRow<ST> R((int)(threadIdx.x / C));
+    const int z0 = (int)(blockIdx.y * planes), z1 = min(z0 + (int)planes, d0);
+    const bool col = cc < nchunk;
+    const bool on1 = g.active[1] != 0, on2 = g.active[2] != 0;
+    const float w1 = on1 ? o1 : 0.f, w2 = on2 ? o2 : 0.f;
+    const bool need_vp = d != 0.f;
+    const size_t pstride = (size_t)d1 * d2 * nchunk;
+    const float4* vc = reinterpret_cast<const float4*>(Vc);
+    // this thread's element (also one past an end of its axis, where it wraps) and, for
+    // the first HALO rows of threads, one element of the halo
+    const int p1 = b1 + R.r1, p2 = b2 + R.r2;
+    const int m1 = axis_at(p1, d1, g.per[1] && on1), m2 = axis_at(p2, d2, g.per[2] && on2);
+    const bool own = col && m1 >= 0 && m2 >= 0;
+    const bool out_row = col && p1 < d1 && p2 < d2;
+    const float4* vown = vc + (own ? ((size_t)m1 * d2 + m2) * nchunk + cc : 0);
+    const int q1 = axis_at(b1 + R.h1, d1, g.per[1] && on1), q2 = axis_at(b2 + R.h2, d2, g.per[2] && on2);
+    const bool hok = R.halo && col && q1 >= 0 && q2 >= 0 && (R.ax1 ? on1 : on2);
+    const float4* vhal = vc + (hok ? ((size_t)q1 * d2 + q2) * nchunk + cc : 0);
+    const uint32_t so = R.own_at() * C + cl, sh = R.halo_at() * C + cl;
+    const uint32_t bufsz = ST::PLANE * C;
+    const float4 zero = vzero(0.f);
+    auto plane = [&](int z, const float4* v, bool ok) {  // (z may be one past either end of axis 0)
+        const int m = axis_at(z, d0, g.per[0] != 0);
+        return ok && m >= 0 ? ldg_stream(v + (size_t)m * pstride) : zero;
+    };
+    const size_t orow = out_row ? (size_t)p1 * d2 + p2 : 0;
+    const float4* vp = reinterpret_cast<const float4*>(Vp) + orow * nchunk + cc;
+    const float* dgp = diag2 + orow;
+    const uint32_t prow = (uint32_t)(d1 * d2);
+    float4* vn = reinterpret_cast<float4*>(Vn) + orow * nchunk + cc;
+    float4 xm = plane(z0 - 1, vown, own), xc = plane(z0, vown, own), xp = plane(z0 + 1, vown, own);
+    float4 hc = plane(z0, vhal, hok), vpc = zero;
+    float dg = 0.f;
+    if (out_row) {
+        if (need_vp) vpc = ldg_stream(vp + (size_t)z0 * pstride);
+        dg = __ldg(dgp + (size_t)z0 * prow);
+    }
+    uint32_t buf = 0;
+    for (int z = z0; z < z1; ++z, buf ^= 1) {
+        // (two buffers: a thread here has passed the barrier of plane z - 1, which every
+        // thread reached after its last read of plane z - 2's buffer)
+        float4* S = sw + buf * bufsz;
+        S[so] = xc;
+        if (R.halo) S[sh] = hc;
+        __syncthreads();
+        // in flight during this plane: plane z + 2, the halo of plane z + 1, V_{k-1} of z + 1
+        float4 xpp = zero, vpn = zero;
+        float dgn = 0.f;
+        if (z + 1 < z1) {
+            xpp = plane(z + 2, vown, own);
+            hc = plane(z + 1, vhal, hok);
+            if (out_row) {
+                if (need_vp) vpn = ldg_stream(vp + (size_t)(z + 1) * pstride);
+                dgn = __ldg(dgp + (size_t)(z + 1) * prow);
+            }
+        }
+        if (out_row) {
+            const float4 s0 = vadd(vadd(zero, xm), xp);
+            float4 s1 = zero, s2 = zero;
+            if (on1) s1 = vadd(vadd(zero, S[so - ST::W2 * C]), S[so + ST::W2 * C]);
+            if (on2) s2 = vadd(vadd(zero, S[so - C]), S[so + C]);
+            float4 acc = vscale(dg, xc);
+            acc = vfma(o0, s0, acc);
+            acc = vfma(w1, s1, acc);
+            acc = vfma(w2, s2, acc);
+            float4 out = vscale(c, acc);
+            if (need_vp) out = vfma(-d, vpc, out);
+            vn[(size_t)z * pstride] = out;
+            if constexpr (PANEL) {
+                const uint32_t i = (uint32_t)((size_t)z * prow + orow);
+                panel_store4(po, i >> 5, i & 31, 4 * cc, out);
+            }
+        }
+        xm = xc;
+        xc = xp;
+        xp = xpp;
+        vpc = vpn;
+        dg = dgn;
+    }
+}
+
 template <typename T, bool PANEL>
 __global__ void __launch_bounds__(512)
 csr_step_kernel(const T* __restrict__ Vc, const T* __restrict__ Vp, T* __restrict__ Vn,
@@ -420,6 +529,36 @@ int panel_grid(uint64_t n_rows) {
 
 }  // namespace
 
+// Launches the sweep kernel where it pays; false where it does not: tiles that do not fit
+// the grid, and blocks below 64 MiB, which the L2 holds (its neighbour reads then cost
+// little, and a run's planes follow one another: 15 to 60 % slower on small grids).
+static bool sweep_step(const StencilGeom& g, int64_t n, uint32_t nchunk, const float* Vc, const float* Vp, float* Vn,
+                       const float* diag2, float o0, float o1, float o2, float c, float d, PanelOut po,
+                       cudaStream_t s) {
+    using ST = Tile3D;
+    if ((uint64_t)n * nchunk * 16 < (64ull << 20)) return false;
+    // chunks a CTA: the fewest idle columns, four on ties
+    uint32_t C = 4, best = ~0u;
+    for (const uint32_t q : {4u, 5u, 6u, 3u, 7u, 8u, 2u, 1u}) {
+        const uint32_t idle = (nchunk + q - 1) / q * q - nchunk;
+        if (idle < best) {
+            best = idle;
+            C = q;
+        }
+    }
+    const uint32_t ngrp = (nchunk + C - 1) / C;
+    // about sixteen 256-thread CTAs an SM over the launch (its last wave is then a small
+    // part), at least eight planes a run
+    const SweepRuns w = sweep_runs<ST>(g.d0, g.d1, g.d2, ngrp, (uint64_t)device_sms() * 16 * 256 / (ST::ROWS * C), 8);
+    if (!w.nseg) return false;
+    const dim3 grid(ngrp * w.nt1 * w.nt2, w.nseg);
+    const size_t smem = (size_t)2 * ST::PLANE * C * 16;
+    const auto kernel = po.base ? stencil_sweep_kernel<true> : stencil_sweep_kernel<false>;
+    kernel<<<grid, ST::ROWS * C, smem, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, g, o0, o1, o2, c, d, nchunk, C, ngrp, w.nt2,
+                                            w.planes, po);
+    return true;
+}
+
 template <typename T>
 static cudaError_t stencil_step(const Plan& P, const T* Vc, const T* Vp, T* Vn, const T* diag2,
                                 T o0, T o1, T o2, T c, T d, uint8_t* panel, cudaStream_t s) {
@@ -456,6 +595,7 @@ static cudaError_t stencil_step(const Plan& P, const T* Vc, const T* Vp, T* Vn, 
                                                                       d, nchunk, (uint32_t)P.n, po);
             return cudaGetLastError();
         }
+        if (sweep_step(P.geom, P.n, nchunk, Vc, Vp, Vn, diag2, o0, o1, o2, c, d, po, s)) return cudaGetLastError();
     }
     if (panel)
         stencil_step_kernel<T, true><<<panel_grid(P.n), stencil_threads(nchunk), 0, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, P.geom, o0,
