@@ -45,7 +45,16 @@
 // accumulators at the start of each interval.  The hand-offs spin on the
 // mbarriers (mbarrier.test_wait).  Every wait is bounded; on expiry the CTA
 // sets bit 2 of the status word and stops.
+//
+// What bounds it: instruction issue in the converting warps and the one-thread MMA loop,
+// not the tensor pipe.  Two values an instruction in the splitting (f32x2), one multiply
+// per two doubled slices, one conversion per drained group instead of shifts on its bits,
+// units dealt round robin over the stages (a stage has fewer than there are threads), and
+// descriptors formed by constant additions: 65536 rows of 200 columns, two Grams a launch,
+// 460 -> ~310 us, the plan's step beside its recurrence 0.51 -> 0.35 ms.
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "internal.h"
 #include "ozslice.cuh"
@@ -59,7 +68,7 @@ using namespace tc;
 using namespace oz;
 
 constexpr int KS = 16;             // rows per stage (one K = 16 MMA step)
-constexpr int FST = 3;             // float64 staging stages
+constexpr int FST = 6;             // most float-pair staging stages (as many as fit, at least 3)
 constexpr int SST = 2;             // slice stages
 constexpr int DRAIN = 20;          // stages between drains: 320 rows
 constexpr int NGRP = 4;            // accumulator groups: i+j = 2, 3, 4, >= 5
@@ -69,6 +78,7 @@ constexpr int NTHREADS = 512;
 constexpr int NCONV = 14;          // converter warps: 2..15
 constexpr int NEPI = 8;            // of which 4..11 also drain the accumulators
 constexpr int MAXN = 256;
+constexpr size_t SMEM_MAX = 222 * 1024;  // dynamic shared memory of a CTA (one an SM)
 constexpr int NBUCKET = 32;        // column-maximum buckets written by the recurrence
 
 __host__ __device__ constexpr int slice_regions(int tile) { return tile == 1 ? 2 * NSL : 2 * NSL - 1; }
@@ -89,15 +99,14 @@ struct OzArgs {
     int ngram;
 };
 
-// Twice each bf16 of a packed 16-byte run (exponent + 1; zeros stay zero).
+// Twice each bf16 of a packed 16-byte run (exact; zeros keep their sign).
 __device__ __forceinline__ uint4 twice8(uint4 a) {
     uint32_t w[4] = {a.x, a.y, a.z, a.w};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        uint32_t lo = w[q] & 0xFFFFu, hi = w[q] >> 16;
-        if (lo & 0x7FFFu) lo += 0x80u;
-        if (hi & 0x7FFFu) hi += 0x80u;
-        w[q] = lo | (hi << 16);
+        __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&w[q]);
+        v = __hmul2(v, __floats2bfloat162_rn(2.f, 2.f));
+        w[q] = *reinterpret_cast<const uint32_t*>(&v);
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
@@ -135,9 +144,11 @@ __device__ __forceinline__ Tile tile_of(int t, int n_tot, int ld, int ntp) {
 // staging of a stage: KS rows of the hi plane, then KS rows of the lo plane, ncopy floats each
 __host__ __device__ inline size_t oz_fstage_bytes(int ncopy) { return (size_t)KS * 2 * ncopy * 4; }
 
-__host__ __device__ inline size_t oz_smem_bytes(int ld) {
-    // worst tile: O (every column copied, two slice sets)
-    return (size_t)FST * oz_fstage_bytes(ld) + (size_t)SST * slice_regions(1) * SLICE_BYTES + 1024;
+// Staging stages beside the slice stages of a tile with nreg slice regions.
+__host__ __device__ inline int oz_fstages(int ld, int nreg) {
+    const size_t room = SMEM_MAX - 1024 - (size_t)SST * nreg * SLICE_BYTES;
+    const int f = (int)(room / oz_fstage_bytes(ld));
+    return f > FST ? FST : f;  // >= 3 for ld <= 256
 }
 
 __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
@@ -146,20 +157,12 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
                  : "r"(taddr));
 }
 
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-}
-
 __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t f_full[FST], f_empty[FST], s_full[SST], s_empty[SST], a_full, a_empty;
     __shared__ uint32_t tmem_slot;
     __shared__ int fail;
-    __shared__ float escale[MAXN];  // 2^-E of each column
+    __shared__ __align__(16) float escale[MAXN];  // 2^-E of each column
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // CTA -> (gram, tile, slab)
@@ -193,8 +196,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
     const size_t fpitch = (size_t)T.ncopy * 4;   // one plane's row (ld floats, a multiple of 16 bytes)
     const size_t fbytes = (size_t)KS * 2 * fpitch;  // hi plane's 16 rows, then the lo plane's
     uint8_t* fbase = smem;
-    uint8_t* sbase = smem + FST * fbytes;
     const int nreg = slice_regions(T.sym ? 0 : 1);
+    const int nf = oz_fstages(P.ld, nreg);
+    uint8_t* sbase = smem + nf * fbytes;
     const size_t sstage = (size_t)nreg * SLICE_BYTES;
 
     // column exponents (max over the buckets of the block's column maxima)
@@ -246,8 +250,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
         if (lane == 0) {  // producer: float-pair rows into the staging ring
             const uint32_t rb = (uint32_t)(T.ncopy * 4);
             for (int q = 0; q < nst; ++q) {
-                const int fs = q % FST;
-                if (q >= FST && !mbar_spin(smem_u32(&f_empty[fs]), ((q / FST) - 1) & 1, &fail)) {
+                const int fs = q % nf;
+                if (q >= nf && !mbar_spin(smem_u32(&f_empty[fs]), ((q / nf) - 1) & 1, &fail)) {
                     atomicOr(&fail, 1);
                     break;
                 }
@@ -264,6 +268,26 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
     } else if (warp == 1) {
         if (lane == 0) {  // MMA issuer
             const uint32_t idesc = instr_desc(T.N);
+            // descriptors of slice 1 in each slice stage; slices and stages are additions to
+            // the address field (16-byte units)
+            const uint64_t base = smem_desc(smem_u32(sbase), 128, GB);
+            uint32_t dg[NGRP];
+#pragma unroll
+            for (int g = 0; g < NGRP; ++g) dg[g] = tmem + (uint32_t)(g * T.N);
+            auto pairs = [&](uint64_t st, uint32_t pos, auto sym) {
+                constexpr bool SYM = decltype(sym)::value;
+#pragma unroll
+                for (int i = 1; i <= NSL; ++i)
+#pragma unroll
+                    for (int j = SYM ? i : 1; i + j <= NSL + 1; ++j) {
+                        const int g = (i + j < 5 ? i + j : 5) - 2;
+                        // slice j: of the other column set, the same one, or its doubled copy
+                        const int rb = !SYM ? NSL + j - 1 : (j == i ? i - 1 : NSL + j - 2);
+                        const bool first = i == 1 && (j < 4 || j == 4);  // of its group in this loop
+                        mma_bf16(dg[g], st + (uint64_t)((i - 1) * (SLICE_BYTES / 16)),
+                                 st + (uint64_t)(rb * (SLICE_BYTES / 16)), idesc, first && pos == 0 ? 0u : 1u);
+                    }
+            };
             bool ok = true;
             for (int q = 0; q < nst && ok; ++q) {
                 const int ss = q % SST, pos = q % DRAIN;
@@ -276,21 +300,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t st = smem_u32(sbase + ss * sstage);
-                uint32_t started = pos != 0 ? 0xFu : 0u;  // groups already holding a sum
-                for (int i = 1; i <= NSL; ++i) {
-                    for (int j = T.sym ? i : 1; i + j <= NSL + 1; ++j) {
-                        const int g = (i + j < 5 ? i + j : 5) - 2;
-                        const uint32_t a = st + (uint32_t)(i - 1) * SLICE_BYTES;
-                        uint32_t b;
-                        if (!T.sym) b = st + (uint32_t)(NSL + j - 1) * SLICE_BYTES;
-                        else if (j == i) b = a;
-                        else b = st + (uint32_t)(NSL + j - 2) * SLICE_BYTES;  // doubled copy of slice j
-                        mma_bf16(tmem + (uint32_t)(g * T.N), smem_desc(a, 128, GB), smem_desc(b, 128, GB), idesc,
-                                 (started >> g) & 1u);
-                        started |= 1u << g;
-                    }
-                }
+                const uint64_t st = base + (uint64_t)(ss * (sstage / 16));
+                if (T.sym)
+                    pairs(st, pos, std::true_type{});
+                else
+                    pairs(st, pos, std::false_type{});
                 umma_commit(&s_empty[ss]);
                 if (pos == DRAIN - 1 || q == nst - 1) umma_commit(&a_full);
             }
@@ -339,10 +353,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     // groups i+j = 2, 3, 4 hold integers in units of 2^-14, 2^-22, 2^-30 (< 2^24 of them)
-                    const long long n2 = float_int(__uint_as_float(v[0][e]) * 16384.0f);
-                    const long long n3 = float_int(__uint_as_float(v[1][e]) * 4194304.0f);
-                    const long long n4 = float_int(__uint_as_float(v[2][e]) * 1073741824.0f);
-                    long long acc = (n2 << 16) + (n3 << 8) + n4;
+                    const int n2 = __float2int_rn(__uint_as_float(v[0][e]) * 16384.0f);
+                    const int n3 = __float2int_rn(__uint_as_float(v[1][e]) * 4194304.0f);
+                    const int n4 = __float2int_rn(__uint_as_float(v[2][e]) * 1073741824.0f);
+                    long long acc = (long long)n2 * 65536 + ((long long)n3 * 256 + n4);
                     float r5 = __uint_as_float(v[3][e]);
                     if (iv > 0) {
                         acc += ((long long)(unsigned)o[e].y << 32) | (unsigned)o[e].x;
@@ -360,16 +374,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
         const int ctid = (warp - 2) * 32 + lane;
         const int ga = T.ga, gt = T.ga + T.gb;
         const int units = KS * gt;
+        const uint32_t rdiv = (65536u + (uint32_t)gt - 1) / (uint32_t)gt;  // u / gt for u < 512
         const int a0 = T.a0, b0 = T.b0, c0 = T.c0, n_tot = P.n_tot;
         const bool sym = T.sym;
         bool alive = true;
+        int fs = 0, fpar = 0, first = ctid;  // staging stage, its parity; first unit of this thread
         for (int q = 0; q < nst; ++q) {
-            const int fs = q % FST, ss = q % SST;
+            const int ss = q % SST;
             if (epi && q > 0 && (q % DRAIN) == 0 && !drain(q / DRAIN - 1)) {
                 alive = false;
                 break;
             }
-            if (!mbar_spin(smem_u32(&f_full[fs]), (q / FST) & 1, &fail)) {
+            if (!mbar_spin(smem_u32(&f_full[fs]), fpar, &fail)) {
                 atomicOr(&fail, 1);
                 alive = false;
                 break;
@@ -384,8 +400,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
             const uint8_t* fst = fbase + fs * fbytes;
             uint8_t* st = sbase + ss * sstage;
             // unit = (row r, 8-column group g): consecutive threads take consecutive groups of
-            // a row (contiguous staging reads, slice stores 272 bytes apart: no bank conflicts)
-            for (int u = ctid; u < units; u += NCONV * 32) {                const int r = u / gt, g = u - r * gt;
+            // a row (contiguous staging reads, slice stores 272 bytes apart: no bank conflicts).
+            // A stage has 256 to 512 units for the 448 converting threads, so each stage starts
+            // where the last one ended: the warps it leaves out go on to the next stage.
+            int u = first;
+            for (; u < units; u += NCONV * 32) {
+                const int r = (int)(((uint32_t)u * rdiv) >> 16), g = u - r * gt;
                 const bool isb = g >= ga;
                 const int gl = isb ? g - ga : g;
                 const int cb = (isb ? b0 : a0) + 8 * gl;  // first global column of the unit
@@ -398,28 +418,29 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
 #pragma unroll
                 for (int h4 = 0; h4 < 2; ++h4) {
                     float4 xh = make_float4(0.f, 0.f, 0.f, 0.f), xl = xh;
+                    const int cc = cb + 4 * h4;
                     if (full) {
                         xh = ph[h4];
                         xl = pl[h4];
                     } else if (row_in) {
                         const float* fh = reinterpret_cast<const float*>(ph) + 4 * h4;
                         const float* fl = reinterpret_cast<const float*>(pl) + 4 * h4;
-                        const int cc = cb + 4 * h4;
                         if (cc + 0 < n_tot) { xh.x = fh[0]; xl.x = fl[0]; }
                         if (cc + 1 < n_tot) { xh.y = fh[1]; xl.y = fl[1]; }
                         if (cc + 2 < n_tot) { xh.z = fh[2]; xl.z = fl[2]; }
                         if (cc + 3 < n_tot) { xh.w = fh[3]; xl.w = fl[3]; }
                     }
-                    const int cc = cb + 4 * h4;
-                    float s0[NSL], s1[NSL], s2[NSL], s3[NSL];
-                    split_df(xh.x, xl.x, escale[cc + 0], s0);
-                    split_df(xh.y, xl.y, escale[cc + 1], s1);
-                    split_df(xh.z, xl.z, escale[cc + 2], s2);
-                    split_df(xh.w, xl.w, escale[cc + 3], s3);
+                    const float4 se = *reinterpret_cast<const float4*>(&escale[cc]);
+                    pair32 s0[NSL], s1[NSL];
+                    split_df2(pair_of(xh.x, xh.y), pair_of(xl.x, xl.y), pair_of(se.x, se.y), s0);
+                    split_df2(pair_of(xh.z, xh.w), pair_of(xl.z, xl.w), pair_of(se.z, se.w), s1);
 #pragma unroll
                     for (int k = 0; k < NSL; ++k) {
-                        w[2 * h4][k] = pack_bf16(s0[k], s1[k]);
-                        w[2 * h4 + 1][k] = pack_bf16(s2[k], s3[k]);
+                        float e0, e1;
+                        pair_get(s0[k], e0, e1);
+                        w[2 * h4][k] = pack_bf16(e0, e1);
+                        pair_get(s1[k], e0, e1);
+                        w[2 * h4 + 1][k] = pack_bf16(e0, e1);
                     }
                 }
                 const size_t inner = (size_t)gl * GB + (r >> 3) * 128 + (r & 7) * 16;
@@ -432,11 +453,16 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
                         *reinterpret_cast<uint4*>(st + (size_t)(NSL + k - 1) * SLICE_BYTES + inner) = twice8(val);
                 }
             }
+            first = u - units;  // < NCONV * 32
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&f_empty[fs]);
                 mbar_arrive(&s_full[ss]);
+            }
+            if (++fs == nf) {
+                fs = 0;
+                fpar ^= 1;
             }
         }
         if (epi && alive && niv > 0) drain(niv - 1);
@@ -649,7 +675,7 @@ cudaError_t launch_gram_oz(const float* Y0, const unsigned long long* cm0, const
     }
     a.cta_per_gram = L.cta_per_gram;
     a.ngram = Y1 ? 2 : 1;
-    const size_t smem = oz_smem_bytes(ld);
+    const size_t smem = SMEM_MAX;
     cudaError_t e = cudaFuncSetAttribute(gram_oz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     gram_oz_kernel<<<a.ngram * L.cta_per_gram, NTHREADS, smem, s>>>(a);

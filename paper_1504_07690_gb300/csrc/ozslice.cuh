@@ -68,6 +68,58 @@ __device__ __forceinline__ void split_df(float hi, float lo, float se, float* s)
     }
 }
 
+// Two float32 in one 64-bit register: sm_100 and later add, multiply and subtract both in one
+// instruction, each rounded as its scalar would be.
+using pair32 = unsigned long long;
+__device__ __forceinline__ pair32 pair_of(float a, float b) {
+    pair32 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ void pair_get(pair32 p, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+__device__ __forceinline__ pair32 pair_add(pair32 a, pair32 b) {
+    pair32 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair32 pair_sub(pair32 a, pair32 b) {
+    pair32 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair32 pair_mul(pair32 a, pair32 b) {
+    pair32 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ pair32 pair_fma(pair32 a, pair32 b, pair32 c) {
+    pair32 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// split_df of two values at once (the same operations, two a instruction).
+__device__ __forceinline__ void split_df2(pair32 hi, pair32 lo, pair32 se, pair32* s) {
+    pair32 r = pair_mul(hi, se);
+    pair32 t = pair_mul(lo, se);
+#pragma unroll
+    for (int k = 1; k <= NSL; ++k) {
+        const float m = __int_as_float((127 + 23 - 7 - 8 * (k - 1)) << 23) * 1.5f;
+        const pair32 M = pair_of(m, m);
+        const pair32 q = pair_sub(pair_add(r, M), M);
+        r = pair_sub(r, q);
+        if (k >= 4) {
+            const pair32 qt = pair_sub(pair_add(t, M), M);
+            t = pair_sub(t, qt);
+            s[k - 1] = pair_add(q, qt);
+        } else {
+            s[k - 1] = q;
+        }
+    }
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&p);
