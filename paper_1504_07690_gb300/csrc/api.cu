@@ -72,6 +72,7 @@ struct ssm_plan_s {
     size_t cap_Et = 0;
     // solver schedule: n_t of the last single-launch solve (its ranks in d_rank), 0 if none
     int32_t* d_perm = nullptr;
+    int32_t* d_pend = nullptr;  // points the warp-per-point solver leaves (small n_v; cap_batch + 1)
     size_t cap_perm = 0;
     int64_t sched_nt = 0;
 };
@@ -327,6 +328,7 @@ void free_plan(ssm_plan_s* h) {
     dev_free(h->d_dos_kpm);
     dev_free(h->d_rank);
     dev_free(h->d_solve);
+    dev_free(h->d_pend);
     dev_free(h->d_tr);
     for (auto e : h->events) cudaEventDestroy(e);
     delete h;
@@ -369,13 +371,17 @@ ssm_status ensure_points(ssm_plan_s* h, int64_t n_t) {
         dev_free(h->d_nu);
         dev_free(h->d_K);
         dev_free(h->d_KZ);
+        dev_free(h->d_pend);
         h->d_mu = h->d_muh = h->d_nu = h->d_K = h->d_KZ = nullptr;
+        h->d_pend = nullptr;
         h->cap_batch = 0;
         CUDA_OR_FAIL(h, dev_alloc(&h->d_mu, (size_t)nb * (M + 1)));
         if (P.p.damping) CUDA_OR_FAIL(h, dev_alloc(&h->d_muh, (size_t)nb * (M + 1)));
         CUDA_OR_FAIL(h, dev_alloc(&h->d_nu, (size_t)nb * (M + 1)));
         CUDA_OR_FAIL(h, dev_alloc(&h->d_K, (size_t)nb * P.n_tot * P.n_tot));
         CUDA_OR_FAIL(h, dev_alloc(&h->d_KZ, (size_t)nb * P.p.n_v * P.p.n_v));
+        if (P.p.n_v <= 32 && P.p.n_vh == 0 && !(P.p.options & SSM_OPT_PINV))
+            CUDA_OR_FAIL(h, dev_alloc(&h->d_pend, (size_t)nb + 1));
         h->cap_batch = nb;
     }
     if (!h->d_zeta) CUDA_OR_FAIL(h, dev_alloc(&h->d_zeta, M + 1));
@@ -529,8 +535,8 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
             // previous such launch, so that the slowest get an SM of their own
             const bool single = t0 == 0 && nb == n_t;
             const int32_t* perm = nullptr;
-            // (no use where every point runs the serial QL chains)
-            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P))) {
+            // (no use where every point runs the serial QL chains, or a warp-size kernel first)
+            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P)) && !h->d_pend) {
                 const int64_t slots = solve_slots(nv, hybrid_routes(P));
                 if (slots >= n_t) {
                     if ((size_t)slots > h->cap_perm) {
@@ -548,7 +554,7 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
             CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, nv, nvh, P.p.tau, xlo, xhi, muh, M + 1, K,
                                          floor_scale, h->d_solve, h->d_dos_ss + t0, h->d_rank + 2 * t0,
                                          P.d_flag, P.stream, nullptr, perm, (P.p.options & SSM_OPT_PINV) != 0,
-                                         hybrid_routes(P)));
+                                         hybrid_routes(P), h->d_pend));
             P.stats.launches++;
             h->sched_nt = single ? n_t : 0;
         }
@@ -787,7 +793,7 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
                                          P.p.damping ? h->d_muh : h->d_mu, M + 1, K, 0.0,
                                          h->d_solve, h->d_dos_ss + b0 * n_tp, h->d_rank + 2 * b0 * n_tp, P.d_flag,
                                          P.stream, h->d_fpt + 3 * b0 * n_tp, nullptr,
-                                         (P.p.options & SSM_OPT_PINV) != 0, hybrid_routes(P)));
+                                         (P.p.options & SSM_OPT_PINV) != 0, hybrid_routes(P), h->d_pend));
             P.stats.launches++;
         }
     }

@@ -346,6 +346,8 @@ cudaError_t launch_asm_oz(const double* coef, int ldc, int64_t n_t, int L, const
                           cudaStream_t s, int64_t tpm = 0, int ne_ld = 0);
 
 // Per-point Alg. 4 + Alg. 6 solve (solve.cu).
+// pend (nullable, n_t + 1 ints): room for the points that the warp-per-point kernel of
+// small n_v leaves to the CTA-per-point one.
 // hyb: hybrid columns take the factored routes (mixed plans with n_vh > 0).
 size_t solve_workspace_bytes(int n_v, bool hyb);
 // floor(t) = floor_scale * sum_{l<=K} (l+1) |mu[t][l]| (see ssm_params.eps_floor).  floor_pt
@@ -354,7 +356,7 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
                          double tau, double xlo, double xhi, const double* mu, int ldmu, int K,
                          double floor_scale, void* work, double* dos, int32_t* rank, int* flag,
                          cudaStream_t s, const double* floor_pt = nullptr, const int32_t* perm = nullptr,
-                         bool pinv = false, bool hyb = false);
+                         bool pinv = false, bool hyb = false, int32_t* pend = nullptr);
 // Resident solver CTAs on the device (SMs x CTAs per SM; 0 if not available): the
 // slots of one wave, the length of a schedule.
 int64_t solve_slots(int n_v, bool hyb);
