@@ -297,6 +297,7 @@ void free_plan(ssm_plan_s* h) {
     dev_free(P.d_slabs);
     dev_free(P.d_slabseg);
     dev_free(P.d_x0max);
+    dev_free(P.d_boff);
     delete[] P.h_row_off;
     delete[] P.h_nb;
     delete[] P.h_ab;
@@ -1038,14 +1039,21 @@ ssm_status moments_batched(ssm_plan_s* h, const double* W, int64_t ldw, double* 
     const size_t nn = (size_t)P.n_tot * P.n_tot, xs = (size_t)(M + 1) * nn;
     ssm_status s = ensure_stage(h, (size_t)P.n * P.n_tot * sizeof(double));
     if (s != SSM_OK) return s;
-    // W (matrices' probe blocks stacked) -> stage with each matrix at its padded row offset
-    CUDA_OR_FAIL(h, cudaMemsetAsync(P.d_stage, 0, (size_t)P.n * P.n_tot * sizeof(double), P.stream));
-    int64_t src = 0;
-    for (int b = 0; b < B; ++b) {
-        CUDA_OR_FAIL(h, cudaMemcpy2DAsync(P.d_stage + (size_t)P.h_row_off[b] * P.n_tot, P.n_tot * sizeof(double),
-                                          W + (size_t)src * ldw, ldw * sizeof(double), P.n_tot * sizeof(double),
-                                          P.h_nb[b], cudaMemcpyDefault, P.stream));
-        src += P.h_nb[b];
+    // W (matrices' probe blocks stacked) -> stage with each matrix at its padded row offset:
+    // one kernel for a device W (a copy per matrix took 4 us each to enqueue), copies from
+    // host memory
+    if (is_device_ptr(W)) {
+        CUDA_OR_FAIL(h, launch_gather_blocks(W, ldw, P.d_boff, B, P.n_tot, P.d_stage, P.stream));
+        P.stats.launches++;
+    } else {
+        CUDA_OR_FAIL(h, cudaMemsetAsync(P.d_stage, 0, (size_t)P.n * P.n_tot * sizeof(double), P.stream));
+        int64_t src = 0;
+        for (int b = 0; b < B; ++b) {
+            CUDA_OR_FAIL(h, cudaMemcpy2DAsync(P.d_stage + (size_t)P.h_row_off[b] * P.n_tot, P.n_tot * sizeof(double),
+                                              W + (size_t)src * ldw, ldw * sizeof(double), P.n_tot * sizeof(double),
+                                              P.h_nb[b], cudaMemcpyHostToDevice, P.stream));
+            src += P.h_nb[b];
+        }
     }
     CUDA_OR_FAIL(h, cudaMemsetAsync(P.d_flag, 0, sizeof(int), P.stream));
     if (!P.graph) {
@@ -1081,20 +1089,10 @@ ssm_status moments_batched(ssm_plan_s* h, const double* W, int64_t ldw, double* 
     if (s != SSM_OK) return s;
     if (flag & 2) return fail(h, SSM_ETIMEOUT, "a tensor-core Gram wait gave up (bounded mbarrier wait)");
     if (flag) return fail(h, SSM_ENONFINITE, "W or the moments contain NaN/Inf");
-    std::vector<double> d0((size_t)B * P.p.n_v), x0(B);
-    for (int b = 0; b < B; ++b)
-        CUDA_OR_FAIL(h, cudaMemcpy2DAsync(d0.data() + (size_t)b * P.p.n_v, sizeof(double), P.d_X + b * xs,
-                                          (P.n_tot + 1) * sizeof(double), sizeof(double), P.p.n_v,
-                                          cudaMemcpyDeviceToHost, P.stream));
+    CUDA_OR_FAIL(h, launch_x0_max(P.d_X, xs, P.n_tot, P.p.n_v, B, P.d_x0max, P.stream));
+    P.stats.launches++;
+    CUDA_OR_FAIL(h, cudaMemcpyAsync(&P.x0max, P.d_x0max, sizeof(double), cudaMemcpyDeviceToHost, P.stream));
     CUDA_OR_FAIL(h, cudaStreamSynchronize(P.stream));
-    for (int b = 0; b < B; ++b) {
-        double m = 0.0;
-        for (int i = 0; i < P.p.n_v; ++i) m = fmax(m, d0[(size_t)b * P.p.n_v + i]);
-        x0[b] = m;
-    }
-    CUDA_OR_FAIL(h, cudaMemcpyAsync(P.d_x0max, x0.data(), B * sizeof(double), cudaMemcpyHostToDevice, P.stream));
-    CUDA_OR_FAIL(h, cudaStreamSynchronize(P.stream));
-    P.x0max = x0[0];
     P.have_moments = true;
     return SSM_OK;
 }
@@ -1551,6 +1549,17 @@ ssm_status ssm_plan_create_batched(ssm_plan_t* out, int32_t B, const ssm_csr* cs
     const size_t nn = (size_t)P.n_tot * P.n_tot;
     BCUDA(dev_alloc(&P.d_X, (size_t)B * (p.degree + 1) * nn));
     BCUDA(dev_alloc(&P.d_x0max, B));
+    {
+        std::vector<int64_t> off(row_off);
+        int64_t src = 0;
+        for (int b = 0; b <= B; ++b) {
+            off.push_back(src);
+            if (b < B) src += nb[b];
+        }
+        BCUDA(dev_alloc(&P.d_boff, off.size()));
+        BCUDA(cudaMemcpyAsync(P.d_boff, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, P.stream));
+        BCUDA(cudaStreamSynchronize(P.stream));  // the host array is a temporary
+    }
     // Gram slabs: each matrix's panels in ~equal slabs, Ge slabs first, then Go
     if (P.use_tc) {
         dev_free(P.d_part_tc);

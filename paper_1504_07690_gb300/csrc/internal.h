@@ -135,6 +135,7 @@ struct Plan {
     int2* d_slabs = nullptr;           // tensor-core Gram slab table [n_e + n_o] (panel ranges)
     int* d_slabseg = nullptr;          // per-matrix slab ranges: se[B+1], so[B+1]
     double* d_x0max = nullptr;         // per-matrix max_i X_0[i][i] (B)
+    int64_t* d_boff = nullptr;         // row_off (B + 1), then the matrices' offsets in W (B + 1)
     cudaStream_t cap_stream = nullptr; // capture streams of the batched recurrence graph (the
     cudaStream_t cap_stream2 = nullptr; // recurrence branch and the Gram branch)
     cudaGraphExec_t graph = nullptr;
@@ -285,6 +286,12 @@ cudaError_t launch_reduce_moments(const double* part, int n_split, int n_tot, do
 cudaError_t launch_check_finite(const double* x, int64_t n, int* flag, cudaStream_t s);
 cudaError_t launch_convert_in(const double* src, int64_t ldsrc, void* dst, int ld, int64_t n_rows,
                               int n_cols, bool to_f32, cudaStream_t s);
+
+// Batched plans: the B stacked probe blocks into their padded rows (off: row offsets (B + 1),
+// then the offsets in W (B + 1)), and the largest diagonal entries of each X_0.
+cudaError_t launch_gather_blocks(const double* W, int64_t ldw, const int64_t* off, int B, int n_cols, double* dst,
+                                 cudaStream_t s);
+cudaError_t launch_x0_max(const double* X, size_t xs, int n_tot, int n_v, int B, double* out, cudaStream_t s);
 
 // Coefficients (coeffs.cu).
 cudaError_t launch_cos_table(double* ctab, int n_theta, cudaStream_t s);

@@ -55,6 +55,33 @@ __global__ void convert_in_kernel(const double* __restrict__ src, int64_t ldsrc,
     }
 }
 
+// Batched plans: the stacked probe blocks W (matrix b's rows from off[B + 1 + b]) -> dst with
+// matrix b's rows from off[b] and zeros up to off[b + 1], n_cols columns.  blockIdx.x walks
+// the matrices, blockIdx.y their rows.
+__global__ void gather_blocks_kernel(const double* __restrict__ W, int64_t ldw, const int64_t* __restrict__ off, int B,
+                                     int n_cols, double* __restrict__ dst) {
+    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+        const int64_t r0 = off[b], s0 = off[B + 1 + b];
+        const int64_t n = off[B + 2 + b] - s0, total = (off[b + 1] - r0) * n_cols;
+        for (int64_t e = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.y * blockDim.x) {
+            const int64_t i = e / n_cols;
+            const int j = (int)(e - i * n_cols);
+            dst[r0 * n_cols + e] = i < n ? W[(s0 + i) * ldw + j] : 0.0;
+        }
+    }
+}
+
+// out[b] = max(0, max_{i < n_v} X_0[i][i]) of matrix b (moments xs values apart); a warp each.
+__global__ void x0_max_kernel(const double* __restrict__ X, size_t xs, int n_tot, int n_v, int B,
+                              double* __restrict__ out) {
+    const int b = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (b >= B) return;
+    double m = 0.0;
+    for (int i = lane; i < n_v; i += 32) m = fmax(m, X[(size_t)b * xs + (size_t)i * (n_tot + 1)]);
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) out[b] = m;
+}
+
 int blocks_for(int64_t n) {
     int64_t b = (n + 255) / 256;
     if (b > (int64_t)device_sms() * 16) b = (int64_t)device_sms() * 16;
@@ -72,6 +99,20 @@ cudaError_t launch_reduce_moments(const double* part, int n_split, int n_tot, do
 
 cudaError_t launch_check_finite(const double* x, int64_t n, int* flag, cudaStream_t s) {
     check_finite_kernel<<<blocks_for(n), 256, 0, s>>>(x, n, flag);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gather_blocks(const double* W, int64_t ldw, const int64_t* off, int B, int n_cols, double* dst,
+                                 cudaStream_t s) {
+    // about 16 CTAs an SM, whether the matrices are many or large
+    const int x = B < 65536 ? B : 65536;
+    int y = (device_sms() * 16 + x - 1) / x;
+    gather_blocks_kernel<<<dim3((unsigned)x, (unsigned)y), 256, 0, s>>>(W, ldw, off, B, n_cols, dst);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_x0_max(const double* X, size_t xs, int n_tot, int n_v, int B, double* out, cudaStream_t s) {
+    x0_max_kernel<<<(unsigned)((B + 7) / 8), 256, 0, s>>>(X, xs, n_tot, n_v, B, out);
     return cudaGetLastError();
 }
 
