@@ -138,18 +138,8 @@ __device__ __forceinline__ void load_item(ItemLoads<T>& L, const RowInfo& ri, ui
     for (int a = 0; a < 3; ++a) {
         const bool lo = (ri.has >> (2 * a)) & 1u, hi = (ri.has >> (2 * a + 1)) & 1u;
         VT sacc = vzero(T(0));
-        if constexpr (sizeof(T) == 8) {
-            // float64 issues at 2 per clock and SM on this part: one add per axis where
-            // both neighbours exist, none otherwise
-            if (lo) sacc = ldg_stream(vc + (size_t)ri.nb[2 * a] * nchunk + cc);
-            if (hi) {
-                const VT h = ldg_stream(vc + (size_t)ri.nb[2 * a + 1] * nchunk + cc);
-                sacc = lo ? vadd(sacc, h) : h;
-            }
-        } else {
-            if (lo) sacc = vadd(sacc, ldg_stream(vc + (size_t)ri.nb[2 * a] * nchunk + cc));
-            if (hi) sacc = vadd(sacc, ldg_stream(vc + (size_t)ri.nb[2 * a + 1] * nchunk + cc));
-        }
+        if (lo) sacc = vadd(sacc, ldg_stream(vc + (size_t)ri.nb[2 * a] * nchunk + cc));
+        if (hi) sacc = vadd(sacc, ldg_stream(vc + (size_t)ri.nb[2 * a + 1] * nchunk + cc));
         L.s[a] = sacc;
     }
     L.vp = need_vp ? ldg_stream(vp + base + cc) : vzero(T(0));
@@ -222,16 +212,9 @@ stencil_step_kernel(const T* __restrict__ Vc, const T* __restrict__ Vp, T* __res
                 VT out = vzero(T(0));
                 if (L[u].ok) {
                     VT acc = vscale(L[u].dg, L[u].x);
-                    if constexpr (sizeof(T) == 8) {  // skip inactive axes and a unit scale
 #pragma unroll
-                        for (int a = 0; a < 3; ++a)
-                            if (g.active[a]) acc = vfma(w[a], L[u].s[a], acc);
-                        out = c == T(1) ? acc : vscale(c, acc);
-                    } else {
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) acc = vfma(w[a], L[u].s[a], acc);
-                        out = vscale(c, acc);
-                    }
+                    for (int a = 0; a < 3; ++a) acc = vfma(w[a], L[u].s[a], acc);
+                    out = vscale(c, acc);
                     if (d != T(0)) out = vfma(-d, L[u].vp, out);
                     vn[(size_t)(pnl * 32 + rr[u]) * nchunk + cq[u]] = out;
                 }
@@ -239,6 +222,48 @@ stencil_step_kernel(const T* __restrict__ Vc, const T* __restrict__ Vp, T* __res
             }
         }
     }
+}
+
+// Float64 stencil step: one (row, 16-byte chunk) item a thread.  Two fmas a clock and SM
+// bound it (6 float64 operations an element on a 2D grid), so what counts is that nothing
+// else takes that pipe (the first step is a flag: comparing c and d would) and that enough
+// warps are there to hide its latency; index arithmetic is free.  On 128 x 128 with 100
+// columns 39 us a step in 32-row panels of 160-thread CTAs (3.4 CTAs an SM), 26 us here
+// (17 us for the operations alone).
+__global__ void __launch_bounds__(256)
+stencil_flat_f64_kernel(const double2* __restrict__ vc, const double2* __restrict__ vp, double2* __restrict__ vn,
+                        const double* __restrict__ diag2, StencilGeom g, double o0, double o1, double o2, double c,
+                        double d, bool first, uint32_t nchunk, uint32_t n_rows) {
+    const uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t i = (uint32_t)(u / nchunk), cc = (uint32_t)(u - (uint64_t)i * nchunk);
+    if (u >= (uint64_t)n_rows * nchunk) return;
+    const size_t at = (size_t)u;
+    const double2 x = __ldg(vc + at);
+    const double dg = __ldg(diag2 + i);
+    double2 p = vzero(0.0);
+    if (!first) p = __ldg(vp + at);
+    const uint32_t i2 = i % g.d2, q = i / g.d2, i1 = q % g.d1, i0 = q / g.d1;
+    const uint32_t co[3] = {i0, i1, i2}, ex[3] = {g.d0, g.d1, g.d2}, sd[3] = {g.d1 * g.d2, g.d2, 1u};
+    double2 lo[3], hi[3];
+    bool has_lo[3], has_hi[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {  // all loads before the first use
+        const uint32_t cm = co[a], e = ex[a], st = sd[a];
+        has_lo[a] = g.active[a] && (cm > 0 || g.per[a]);
+        has_hi[a] = g.active[a] && (cm + 1 < e || g.per[a]);
+        lo[a] = hi[a] = vzero(0.0);
+        if (has_lo[a]) lo[a] = __ldg(vc + (size_t)(cm > 0 ? i - st : i + (e - 1) * st) * nchunk + cc);
+        if (has_hi[a]) hi[a] = __ldg(vc + (size_t)(cm + 1 < e ? i + st : i - (e - 1) * st) * nchunk + cc);
+    }
+    const double w[3] = {o0, o1, o2};
+    double2 acc = vscale(dg, x);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        if (g.active[a]) {
+            const double2 s = !has_hi[a] ? lo[a] : (has_lo[a] ? vadd(lo[a], hi[a]) : hi[a]);
+            acc = vfma(w[a], s, acc);
+        }
+    vn[at] = first ? vscale(c, acc) : vfma(-d, p, acc);  // c = 1 after the first step
 }
 
 // Float32 stencil step on grids whose axis 0 is inactive (2D and 1D grids): a thread
@@ -559,12 +584,11 @@ static bool sweep_step(const StencilGeom& g, int64_t n, uint32_t nchunk, const f
     return true;
 }
 
-template <typename T>
-static cudaError_t stencil_step(const Plan& P, const T* Vc, const T* Vp, T* Vn, const T* diag2,
-                                T o0, T o1, T o2, T c, T d, uint8_t* panel, cudaStream_t s) {
-    const uint32_t nchunk = (uint32_t)(P.ld / Vec16<T>::W);
+static cudaError_t stencil_step_f32(const Plan& P, const float* Vc, const float* Vp, float* Vn, const float* diag2,
+                                    float o0, float o1, float o2, float c, float d, uint8_t* panel, cudaStream_t s) {
+    const uint32_t nchunk = (uint32_t)(P.ld / Vec16<float>::W);
     const PanelOut po{panel, (uint32_t)P.panel_groups};
-    if constexpr (sizeof(T) == 4) {
+    {
         // Trailing axes of extent 1 (always inactive) change no row index: (d0, d1, 1) is
         // the grid (1, d0, d1).  With axis 0 then inactive (2D and 1D grids) the row-group
         // kernel runs, marching along the unit-stride axis (5 loads a row instead of 6).
@@ -597,12 +621,9 @@ static cudaError_t stencil_step(const Plan& P, const T* Vc, const T* Vp, T* Vn, 
         }
         if (sweep_step(P.geom, P.n, nchunk, Vc, Vp, Vn, diag2, o0, o1, o2, c, d, po, s)) return cudaGetLastError();
     }
-    if (panel)
-        stencil_step_kernel<T, true><<<panel_grid(P.n), stencil_threads(nchunk), 0, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, P.geom, o0,
-                                                                        o1, o2, c, d, nchunk, (uint32_t)P.n, po);
-    else
-        stencil_step_kernel<T, false><<<panel_grid(P.n), stencil_threads(nchunk), 0, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, P.geom, o0,
-                                                                         o1, o2, c, d, nchunk, (uint32_t)P.n, po);
+    const auto kernel = panel ? stencil_step_kernel<float, true> : stencil_step_kernel<float, false>;
+    kernel<<<panel_grid(P.n), stencil_threads(nchunk), 0, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, P.geom, o0, o1, o2, c, d,
+                                                               nchunk, (uint32_t)P.n, po);
     return cudaGetLastError();
 }
 
@@ -625,11 +646,17 @@ static cudaError_t csr_step(const Plan& P, const T* Vc, const T* Vp, T* Vn, cons
 
 cudaError_t launch_stencil_step_f64(const Plan& P, const double* Vc, const double* Vp, double* Vn,
                                     double c, double d, cudaStream_t s) {
-    return stencil_step<double>(P, Vc, Vp, Vn, P.d_diag64, P.off64[0], P.off64[1], P.off64[2], c, d, nullptr, s);
+    if (d != 0.0 && c != 1.0) return cudaErrorInvalidValue;  // (1/2, 0) or (1, 1)
+    const uint32_t nchunk = (uint32_t)(P.ld / 2);
+    const uint64_t blocks = ((uint64_t)P.n * nchunk + 255) / 256;
+    stencil_flat_f64_kernel<<<(unsigned)blocks, 256, 0, s>>>(
+        (const double2*)Vc, (const double2*)(Vp ? Vp : Vc), (double2*)Vn, P.d_diag64, P.geom, P.off64[0], P.off64[1],
+        P.off64[2], c, d, d == 0.0, nchunk, (uint32_t)P.n);
+    return cudaGetLastError();
 }
 cudaError_t launch_stencil_step_f32(const Plan& P, const float* Vc, const float* Vp, float* Vn,
                                     float c, float d, uint8_t* panel, cudaStream_t s) {
-    return stencil_step<float>(P, Vc, Vp, Vn, P.d_diag32, P.off32[0], P.off32[1], P.off32[2], c, d, panel, s);
+    return stencil_step_f32(P, Vc, Vp, Vn, P.d_diag32, P.off32[0], P.off32[1], P.off32[2], c, d, panel, s);
 }
 cudaError_t launch_csr_step_f64(const Plan& P, const double* Vc, const double* Vp, double* Vn,
                                 double c, double d, cudaStream_t s) {
