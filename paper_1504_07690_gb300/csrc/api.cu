@@ -537,7 +537,8 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
             const bool single = t0 == 0 && nb == n_t;
             const int32_t* perm = nullptr;
             // (no use where every point runs the serial QL chains, or a warp-size kernel first)
-            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P)) && !h->d_pend) {
+            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P)) &&
+                !solve_uses_small(n_t, nv, nvh, (P.p.options & SSM_OPT_PINV) != 0)) {
                 const int64_t slots = solve_slots(nv, hybrid_routes(P));
                 if (slots >= n_t) {
                     if ((size_t)slots > h->cap_perm) {

@@ -106,7 +106,7 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
     if (grid > n_slot) grid = n_slot;
     // small points without hybrid columns: a warp each; what is left goes on
     const int32_t* n_dev = nullptr;
-    if (pend && n_v <= SOLVE_SMALL_N && n_vh == 0 && !pinv) {
+    if (pend && solve_uses_small(n_t, n_v, n_vh, pinv)) {
         e = launch_solve_small(Kfull, KZ, n_t, n_v, tau, xlo, xhi, mu, ldmu, K, floor_scale, dos, rank, floor_pt, pend,
                                s);
         if (e != cudaSuccess) return e;
@@ -117,6 +117,14 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
                                                    floor_scale, (double*)work, dos, rank, flag, floor_pt, perm,
                                                    n_slot, pinv, n_dev);
     return cudaGetLastError();
+}
+
+// A warp a point when the points fill the device with warps; fewer take one wave of CTAs
+// either way, and a warp's serial chain is the longer one (n_v = 32: 1.06 against 1.31 ms
+// at 73 points, 1.19 against 1.34 at 600, 1.79 against 1.44 at 1200; n_v = 16: 0.42
+// against 0.55, 0.60 against 0.59, 0.72 against 0.65).
+bool solve_uses_small(int64_t n_t, int n_v, int n_vh, bool pinv) {
+    return n_v <= SOLVE_SMALL_N && n_vh == 0 && !pinv && n_t >= (int64_t)8 * device_sms();
 }
 
 int64_t solve_slots(int n_v, bool hyb) {
