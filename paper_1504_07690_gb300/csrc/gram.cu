@@ -20,7 +20,7 @@ namespace {
 
 constexpr int KT = 32;  // rows per staged slab
 
-// Tile shapes.  A warp owns one square piece of the tile, 8 x 4 lanes of P x Q outputs,
+// Tile shapes.  A warp owns one 8 P x 4 Q piece of the tile, 8 x 4 lanes of P x Q outputs,
 // and sums each output over the slice's rows in row order (one fma chain per output), so
 // the shape changes no bit of the result.  Float64 runs at 2 fma a clock and SM here: the
 // kernel is bound by the fma pipe (97 % busy), and what counts is that no warp multiplies
@@ -32,14 +32,25 @@ constexpr int KT = 32;  // rows per staged slab
 //   Mid, Small: one warp a tile, 16 x 16 and 8 x 8, for problems with few tiles and
 //     slices (1024 rows x 40 columns: 545 us in two slices of 64 x 64 tiles, that is on
 //     four SMs).
-// ST: staged slabs (more than two did not help the one-warp tiles: 8.5 against 8.3 ms a
-// call of the 32 x 32 grid, 40 probes, degree 200).
+// ST: staged slabs (more than two did not help the one-warp tiles).  Staged with 16-byte
+// copies where rows are whole 16-byte units: 7.2 ms a call of the 32 x 32 grid, 40 probes,
+// degree 200, against 7.7 with 8-byte ones.
 struct WideTile { static constexpr int P = 2, Q = 4, WR = 2, WC = 2, ST = 2; };
 struct MidTile { static constexpr int P = 2, Q = 4, WR = 1, WC = 1, ST = 2; };
 struct SmallTile { static constexpr int P = 1, Q = 2, WR = 1, WC = 1, ST = 2; };
 
-template <typename S> constexpr int piece() { return 8 * S::P; }
-template <typename S> constexpr int tile_dim() { return piece<S>() * S::WR; }
+template <typename S>
+constexpr int tile_dim() {
+    static_assert(8 * S::P * S::WR == 4 * S::Q * S::WC, "square tiles");
+    return 8 * S::P * S::WR;
+}
+
+// 16 aligned bytes, of which the first `bytes` are read and the others zero.
+__device__ __forceinline__ void async_vec(void* dst, const void* src, int bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(bytes)
+                 : "memory");
+}
 
 template <typename T>
 __device__ __forceinline__ void async_elem(T* dst, const T* src, bool ok) {
@@ -49,8 +60,7 @@ __device__ __forceinline__ void async_elem(T* dst, const T* src, bool ok) {
                  : "memory");
 }
 
-// Tile u of the nt1 x nt1 tiles of G^o (which = 1) and the upper ones of G^e, the full
-// tiles before the ragged ones (the light CTAs fill the tail of the launch).
+// Tile u of the nt1 x nt1 tiles of G^o (which = 1), then the upper ones of G^e.
 __device__ __forceinline__ void tile_of_index(int u, int nt1, int n_sym, int& which, int& ti, int& tj) {
     const int n_all = nt1 * nt1;
     const bool odd = (int)gridDim.x > n_sym;
@@ -73,8 +83,8 @@ __device__ __forceinline__ void tile_of_index(int u, int nt1, int n_sym, int& wh
 template <typename T, typename Acc, typename S>
 __global__ void __launch_bounds__(32 * S::WR * S::WC)
 gram_kernel(const T* __restrict__ A, const T* __restrict__ B, int ld, int n_tot, int64_t n_rows,
-            int64_t rows_per_split, double* __restrict__ part, int nt1, int n_sym) {
-    constexpr int NT = 32 * S::WR * S::WC, TD = tile_dim<S>(), PD = piece<S>(), P = S::P, Q = S::Q;
+            int64_t rows_per_split, double* __restrict__ part, int nt1, int n_sym, bool vec) {
+    constexpr int NT = 32 * S::WR * S::WC, TD = tile_dim<S>(), P = S::P, Q = S::Q, PR = 8 * P, PC = 4 * Q;
     __shared__ __align__(16) T Ls[S::ST][KT][TD];
     __shared__ __align__(16) T Rs[S::ST][KT][TD];
     int which, ti, tj;
@@ -86,15 +96,37 @@ gram_kernel(const T* __restrict__ A, const T* __restrict__ B, int ld, int n_tot,
     if (r1 > n_rows) r1 = n_rows;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int cl0 = ti * TD, cr0 = tj * TD;
-    const int pr = (warp / S::WC) * PD, pc = (warp % S::WC) * PD;  // the warp's piece of the tile
-    const bool on = cl0 + pr < n_tot && cr0 + pc < n_tot && (which == 1 || cr0 + pc + PD > cl0 + pr);
+    const int pr = (warp / S::WC) * PR, pc = (warp % S::WC) * PC;  // the warp's piece of the tile
+    const bool on = cl0 + pr < n_tot && cr0 + pc < n_tot && (which == 1 || cr0 + pc + PC > cl0 + pr);
     const int ri = pr + (lane >> 2) * P, ci = pc + (lane & 3) * Q;
     Acc acc[P][Q];
 #pragma unroll
     for (int p = 0; p < P; ++p)
 #pragma unroll
         for (int q = 0; q < Q; ++q) acc[p][q] = Acc(0);
+    // 16-byte copies (vec: rows of aligned 16-byte units): a thread keeps one unit column of
+    // both tiles and steps over the rows
+    constexpr int VE = 16 / (int)sizeof(T), VC = TD / VE, VR = NT / VC;
+    const int vr = (int)threadIdx.x / VC, vc = ((int)threadIdx.x % VC) * VE;
+    const int vl = max(0, min(VE, n_tot - cl0 - vc)) * (int)sizeof(T);  // bytes of the unit in the row
+    const int vq = max(0, min(VE, n_tot - cr0 - vc)) * (int)sizeof(T);
+    const T* Lv = L + (vl ? cl0 + vc : 0);
+    const T* Rv = R + (vq ? cr0 + vc : 0);
     auto stage = [&](int buf, int64_t r) {  // rows r .. r + KT - 1 (an empty group past the slice)
+        if (vec) {
+            if (r < r1) {
+                const size_t o = (size_t)(r + vr) * ld;
+#pragma unroll
+                for (int q = 0; q < KT / VR; ++q) {
+                    const bool in = r + vr + q * VR < r1;
+                    const size_t at = in ? o + (size_t)q * VR * ld : 0;
+                    async_vec(&Ls[buf][vr + q * VR][vc], Lv + at, in ? vl : 0);
+                    async_vec(&Rs[buf][vr + q * VR][vc], Rv + at, in ? vq : 0);
+                }
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            return;
+        }
         for (int e = threadIdx.x; e < KT * TD && r < r1; e += NT) {
             const int rr = e / TD, cc = e - rr * TD;
             const int64_t row = r + rr;
@@ -150,7 +182,8 @@ cudaError_t gram_launch(const T* A, const T* B, int ld, int n_tot, int64_t n_row
     const int nt1 = (n_tot + tile_dim<S>() - 1) / tile_dim<S>();
     const int n_sym = nt1 * (nt1 + 1) / 2;
     dim3 grid((unsigned)(n_sym + (B ? nt1 * nt1 : 0)), (unsigned)n_split);
-    gram_kernel<T, Acc, S><<<grid, 32 * S::WR * S::WC, 0, s>>>(A, B, ld, n_tot, n_rows, rps, part, nt1, n_sym);
+    const bool vec = ld % (16 / (int)sizeof(T)) == 0 && ((uintptr_t)A & 15) == 0 && ((uintptr_t)B & 15) == 0;
+    gram_kernel<T, Acc, S><<<grid, 32 * S::WR * S::WC, 0, s>>>(A, B, ld, n_tot, n_rows, rps, part, nt1, n_sym, vec);
     return cudaGetLastError();
 }
 
