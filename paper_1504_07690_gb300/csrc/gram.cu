@@ -29,15 +29,18 @@ constexpr int KT = 32;  // rows per staged slab
 //     diagonal idle.  The Gram pair of two 65536 x 200 float64 blocks: 8.05 ms, 13.7 ms
 //     with 64 x 64 tiles computed whole (1.77 times the useful products; 6.3 ms is the
 //     pipe's floor for these alone).
-//   Mid, Small: one warp a tile, 16 x 16 and 8 x 8, for problems with few tiles and
-//     slices (1024 rows x 40 columns: 545 us in two slices of 64 x 64 tiles, that is on
-//     four SMs).
-// ST: staged slabs (more than two did not help the one-warp tiles).  Staged with 16-byte
+//   Mid: one warp a 16 x 16 tile, for problems with few tiles and slices.
+//   Small: 8 x 8 tiles of two warps, one output a lane, for the smallest: an fma holds its
+//     warp for 65 to 73 cycles whatever the others do, so a lane's second output would double
+//     the chain of a slice (1024 rows x 40 columns in two slices of 512 rows: 545 us in
+//     64 x 64 tiles, on four SMs; 43 us with two outputs a lane, 28 us with one, launch
+//     included).
+// ST: staged slabs (more than two did not help the small tiles).  Staged with 16-byte
 // copies where rows are whole 16-byte units: 7.2 ms a call of the 32 x 32 grid, 40 probes,
-// degree 200, against 7.7 with 8-byte ones.
+// degree 200, against 7.7 with 8-byte ones (both with two outputs a lane).
 struct WideTile { static constexpr int P = 2, Q = 4, WR = 2, WC = 2, ST = 2; };
 struct MidTile { static constexpr int P = 2, Q = 4, WR = 1, WC = 1, ST = 2; };
-struct SmallTile { static constexpr int P = 1, Q = 2, WR = 1, WC = 1, ST = 2; };
+struct SmallTile { static constexpr int P = 1, Q = 1, WR = 1, WC = 2, ST = 2; };
 
 template <typename S>
 constexpr int tile_dim() {
