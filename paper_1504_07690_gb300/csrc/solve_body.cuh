@@ -683,19 +683,86 @@ __device__ void bisect_all(int n, Shared& sh) {
     __syncthreads();
 }
 
+// One row of 16 columns solved against the 16 x 16 lower triangle of t (ld 33, from row and
+// column c0): s[c] = (s[c] - sum_{m < c} s[m] t[c][m]) rd[c], right-looking, so that the
+// updates of one step are independent (a float64 fma takes 73 cycles and issues in 16; each
+// s[c] still subtracts its terms in order of m).
+__device__ __forceinline__ void solve_row16(double (&s)[16], const double* t, const double* rd) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        s[c] *= rd[c];
+#pragma unroll
+        for (int j = c + 1; j < 16; ++j) s[j] = fma(-s[c], t[j * 33 + c], s[j]);
+    }
+}
+
+// 16 columns of a Cholesky on one warp, right-looking in registers: lane `top + c` holds the
+// pivot row of column c, s[0..15] the columns of every lane's row from the pivot rows down.
+// rd[c] = 1 / L[c][c] for c < w.  False (on every lane) at the first pivot that is not positive.
+__device__ __forceinline__ bool factor_cols16(double (&s)[16], int top, int w, double* rd, int lane) {
+    bool pos = true;
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+        if (c < w && pos) {
+            const double piv = __shfl_sync(0xffffffffu, s[c], top + c);
+            pos = piv > 0.0;
+            const double r0 = rsqrt(piv);
+            const double rr = r0 * fma(-0.5 * piv * r0, r0, 1.5);  // one Newton step
+            if (lane == 0) rd[c] = rr;
+            const double l = (lane == top + c ? piv : s[c]) * rr;
+            s[c] = l;
+#pragma unroll
+            for (int j = c + 1; j < 16; ++j) {
+                const double lj = __shfl_sync(0xffffffffu, l, top + j);
+                s[j] = fma(-l, lj, s[j]);
+            }
+        }
+    return pos;
+}
+
+// Cholesky of the w x w block ta (ld 33, w <= 32) on one warp, lane = row: its lower triangle
+// into td (ld 33), the inverses of its diagonal into rd.  Rows stay in registers, 16 columns
+// at a time (in shared memory each update waited for the one before it).
+__device__ __forceinline__ bool factor_diag(const double* ta, double* td, double* rd, int w, int lane) {
+    double s[16];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) s[c] = lane < w && c < w ? ta[lane * 33 + c] : 0.0;
+    if (!factor_cols16(s, 0, w, rd, lane)) return false;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) td[lane * 33 + c] = s[c];
+    if (w <= 16) return true;
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 16; ++c) s[c] = lane < w && 16 + c < w ? ta[lane * 33 + 16 + c] : 0.0;
+#pragma unroll 4
+    for (int m = 0; m < 16; ++m) {
+        const double x = td[lane * 33 + m];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) s[c] = fma(-x, td[(16 + c) * 33 + m], s[c]);
+    }
+    if (!factor_cols16(s, 16, w - 16, rd + 16, lane)) return false;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) td[lane * 33 + 16 + c] = s[c];
+    __syncwarp();
+    return true;
+}
+
 // Cholesky factor of the symmetric positive definite n x n matrix A
 // (row-major): the lower triangle of A receives L (A = L L^T) and sh.v[k] =
 // 1 / L[k][k].  Returns false (on every thread) at the first pivot that is not
 // positive.  Blocked, left-looking, panels of 32 columns: each 32-row tile of
 // the panel is formed as A - L[:, :jb] L[panel, :jb]^T from 32 x 32 tiles
 // staged in shared memory (2 x 2 outputs per thread, as gemm_tn); the diagonal
-// block is then factored in shared memory by one warp (one row per lane), and
-// the tiles below it are solved against it (L = C L_D^-T) by one warp, also in
-// shared memory.  Only L's finished columns are read from global memory, once
-// per panel, instead of a read-modify-write of the whole trailing matrix for
-// every column.
-__device__ bool cholesky_lower(double* __restrict__ A, int n, Shared& sh) {
-    double* ta = sh.gt;            // [32][33]: staged L rows of the tile, then the tile itself
+// block is factored in shared memory by one warp (one row per lane), and
+// then the tiles below it are solved against it (L = C L_D^-T), a warp a tile, a row a
+// lane, 16 columns at a time in registers.  Only L's finished columns are read from global
+// memory, once per panel, instead of a read-modify-write of the whole trailing matrix for
+// every column.  Not inlined: nine calls of the solve share it.  The diagonal block's
+// chain of 32 columns is what the panels wait for: with its columns in registers (factor_diag)
+// and the tiles below solved by all warps, 16 points of n_v = 128 take 1.69 ms, 2.17 with the
+// block and the row solves in shared memory.
+__device__ __noinline__ bool cholesky_lower(double* __restrict__ A, int n, const Shared& sh) {
+    double* ta = sh.gt;            // [32][33]: staged L rows of the tile, then the diagonal tile
     double* tb = sh.gt + 32 * 33;  // [32][33]: staged L rows of the panel
     double* td = tb + 32 * 33;     // [32][33]: factored diagonal block L_D
     const int tid = threadIdx.x, nt = (int)blockDim.x, warp = tid >> 5, lane = tid & 31;
@@ -730,8 +797,22 @@ __device__ bool cholesky_lower(double* __restrict__ A, int n, Shared& sh) {
                     }
                 }
             }
+            if (i0 > jb) {
+                // the updated tile C = A[i0.., jb..] - acc in place, solved below
+                if (jb > 0)
+#pragma unroll
+                    for (int pass = 0; pass < 4; ++pass) {
+                        const int t = tid + pass * nt;
+                        const int pi = 2 * (t >> 4), qj = 2 * (t & 15);
+                        for (int i = 0; i < 2; ++i)
+                            for (int j = 0; j < 2; ++j)
+                                if (t < 256 && pi + i < h && qj + j < w)
+                                    A[(size_t)(i0 + pi + i) * n + jb + qj + j] -= acc[pass][i][j];
+                    }
+                continue;
+            }
             __syncthreads();
-            // the updated tile C = A[i0.., jb..] - acc into ta[row][col]
+            // the diagonal tile into ta[row][col]
 #pragma unroll
             for (int pass = 0; pass < 4; ++pass) {
                 const int t = tid + pass * nt;
@@ -745,56 +826,41 @@ __device__ bool cholesky_lower(double* __restrict__ A, int n, Shared& sh) {
                 }
             }
             __syncthreads();
-            if (i0 == jb) {
-                // diagonal block: right-looking in shared memory, lane = row
-                if (warp == 0) {
-                    bool pos = true;
-                    for (int c = 0; c < w && pos; ++c) {
-                        const double piv = ta[c * 33 + c];
-                        pos = piv > 0.0;
-                        if (!pos) break;
-                        const double r0 = rsqrt(piv);
-                        const double rr = r0 * fma(-0.5 * piv * r0, r0, 1.5);  // one Newton step
-                        if (lane == 0) sh.v[jb + c] = rr;
-                        __syncwarp();
-                        if (lane == c) ta[c * 33 + c] = piv * rr;
-                        if (lane > c && lane < w) ta[lane * 33 + c] *= rr;
-                        __syncwarp();
-                        if (lane > c && lane < w) {
-                            const double lic = ta[lane * 33 + c];
-                            for (int j = c + 1; j <= lane; ++j) ta[lane * 33 + j] = fma(-lic, ta[j * 33 + c], ta[lane * 33 + j]);
-                        }
-                        __syncwarp();
-                    }
-                    if (lane == 0) sh.misc[6] = pos;
-                }
-                __syncthreads();
-                if (!sh.misc[6]) return false;
-                for (int e = tid; e < 32 * 32; e += nt) {
-                    const int ii = e >> 5, c = e & 31;
-                    if (ii < w && c <= ii) {
-                        const double v = ta[ii * 33 + c];
-                        td[ii * 33 + c] = v;
-                        A[(size_t)(jb + ii) * n + jb + c] = v;
-                    }
-                }
-            } else {
-                // rows below the diagonal block: forward substitution, lane = row
-                if (warp == 0 && lane < h) {
-                    for (int c = 0; c < w; ++c) {
-                        double s = ta[lane * 33 + c];
-                        for (int m = 0; m < c; ++m) s = fma(-ta[lane * 33 + m], td[c * 33 + m], s);
-                        ta[lane * 33 + c] = s * sh.v[jb + c];
-                    }
-                }
-                __syncthreads();
-                for (int e = tid; e < 32 * 32; e += nt) {
-                    const int ii = e >> 5, c = e & 31;
-                    if (ii < h && c < w) A[(size_t)(i0 + ii) * n + jb + c] = ta[ii * 33 + c];
-                }
+            if (warp == 0) {
+                const bool pos = factor_diag(ta, td, sh.v + jb, w, lane);
+                if (lane == 0) sh.misc[6] = pos;
             }
             __syncthreads();
+            if (!sh.misc[6]) return false;
+            for (int e = tid; e < 32 * 32; e += nt) {
+                const int ii = e >> 5, c = e & 31;
+                if (ii < w && c <= ii) A[(size_t)(jb + ii) * n + jb + c] = td[ii * 33 + c];
+            }
         }
+        // the tiles below the diagonal block (the last panel has none, so w = 32 here)
+        __syncthreads();
+        for (int i = jb + 32 * (warp + 1) + lane; i - lane < n; i += nt) {
+            if (i >= n) continue;
+            double* row = A + (size_t)i * n + jb;
+            double s[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) s[c] = row[c];
+            solve_row16(s, td, sh.v + jb);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) row[c] = s[c];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) s[c] = row[16 + c];
+#pragma unroll 4
+            for (int m = 0; m < 16; ++m) {
+                const double x = row[m];
+#pragma unroll
+                for (int c = 0; c < 16; ++c) s[c] = fma(-x, td[(16 + c) * 33 + m], s[c]);
+            }
+            solve_row16(s, td + 16 * 33 + 16, sh.v + jb + 16);
+#pragma unroll
+            for (int c = 0; c < 16; ++c) row[16 + c] = s[c];
+        }
+        __syncthreads();
     }
     return true;
 }
