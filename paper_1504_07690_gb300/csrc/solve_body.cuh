@@ -55,6 +55,9 @@ constexpr int MAXN = 1024;       // largest n_v
 constexpr int MAX_QL_ITER = 60;
 constexpr int BT_CHUNKS = 8;     // columns a lane keeps in registers in back_transform: 32 x 8
 
+// The larger functions of the factored routes are not inlined: a point runs through most of
+// them once, and inlined at every call they missed the instruction cache (400 points of
+// n_v = 200: 20.2 ms inlined, 19.5 as they are).
 struct Shared {
     double* d;     // n: diagonal, then eigenvalues
     double* off;   // n: off-diagonal T[i][i+1]
@@ -521,7 +524,7 @@ __device__ bool ql_implicit(double* __restrict__ Zt, int n, bool vectors, Shared
 // p_{i-1}).  The pair (p_i, p_{i-1}) is rescaled by 2^-/+600 when p_i leaves
 // [2^-600, 2^600].  Signs and exponent tests use the integer pipe (the
 // float64 pipe runs at 1/58 of the float32 rate on this part).
-__device__ int sturm_below(const double* __restrict__ d, const double* __restrict__ e2, int n, double x) {
+__device__ __noinline__ int sturm_below(const double* __restrict__ d, const double* __restrict__ e2, int n, double x) {
     double pm = 1.0, pc = d[0] - x;
     int neg_prev = 0, count = 0;
     for (int i = 0;; ++i) {
@@ -546,7 +549,7 @@ __device__ int sturm_below(const double* __restrict__ d, const double* __restric
 
 // Same count in float32 for the coarse part of the bisection (the sequence
 // is rescaled by 2^-/+60 to stay inside the float32 range).
-__device__ int sturm_below_f32(const float* __restrict__ d, const float* __restrict__ e2, int n, float x) {
+__device__ __noinline__ int sturm_below_f32(const float* __restrict__ d, const float* __restrict__ e2, int n, float x) {
     float pm = 1.f, pc = d[0] - x;
     int neg_prev = 0, count = 0;
     for (int i = 0;; ++i) {
@@ -577,7 +580,7 @@ __device__ int sturm_below_f32(const float* __restrict__ d, const float* __restr
 // eigenvalue is certain to lie within a few float32 ulps of the float32
 // bracket, so the bracket is widened by 8 ulps of its magnitude before the
 // float64 pass), then refined in float64.
-__device__ void bisect_prepare(int n, Shared& sh) {
+__device__ __noinline__ void bisect_prepare(int n, Shared& sh) {
     const int tid = threadIdx.x;
     float* d32 = reinterpret_cast<float*>(sh.rs);
     float* e32 = d32 + n;
@@ -867,7 +870,7 @@ __device__ __noinline__ bool cholesky_lower(double* __restrict__ A, int n, const
 
 // X <- L^{-1} X for the n x n row-major X, L from cholesky_lower (rdiag =
 // sh.v): forward substitution, one column of X per thread.
-__device__ void trsm_lower(const double* __restrict__ L, double* __restrict__ X, int n, const Shared& sh) {
+__device__ __noinline__ void trsm_lower(const double* __restrict__ L, double* __restrict__ X, int n, const Shared& sh) {
     for (int c = threadIdx.x; c < n; c += (int)blockDim.x) {
         for (int i = 0; i < n; ++i)
             X[(size_t)i * n + c] = (X[(size_t)i * n + c] - dot8(L + (size_t)i * n, 1, X + c, n, i)) * sh.v[i];
@@ -877,7 +880,7 @@ __device__ void trsm_lower(const double* __restrict__ L, double* __restrict__ X,
 
 // Y <- L^{-1} X^T (X, Y distinct, n x n row-major): forward substitution on
 // the rows of X, one row per thread; row r of X gives column r of Y.
-__device__ void trsm_lower_t(const double* __restrict__ L, const double* __restrict__ X, double* __restrict__ Y,
+__device__ __noinline__ void trsm_lower_t(const double* __restrict__ L, const double* __restrict__ X, double* __restrict__ Y,
                              int n, const Shared& sh) {
     for (int r = threadIdx.x; r < n; r += (int)blockDim.x) {
         const double* xr = X + (size_t)r * n;
@@ -891,7 +894,7 @@ __device__ void trsm_lower_t(const double* __restrict__ L, const double* __restr
 // X overwrites it), L from cholesky_lower (rdiag = sh.v).  X is lower triangular
 // as well, so column c is a forward substitution from row c down (n^3 / 3 flops),
 // one column per thread.
-__device__ double trtr_sumsq(const double* __restrict__ L, double* __restrict__ M, int n, const Shared& sh) {
+__device__ __noinline__ double trtr_sumsq(const double* __restrict__ L, double* __restrict__ M, int n, const Shared& sh) {
     double f = 0.0;
     for (int c = threadIdx.x; c < n; c += (int)blockDim.x) {
         for (int i = c; i < n; ++i) {
@@ -913,7 +916,7 @@ __device__ double trtr_sumsq(const double* __restrict__ L, double* __restrict__ 
 // interval (the subtraction would cancel), the eigenvalues inside are found
 // and summed in index order instead.  sh.misc[2], sh.misc[3]: the index range [jl, jh) of
 // the eigenvalues inside.
-__device__ double range_sum(double* __restrict__ C, int m, double xl, double xh, Shared& sh, int* count) {
+__device__ __noinline__ double range_sum(double* __restrict__ C, int m, double xl, double xh, Shared& sh, int* count) {
     const int tid = threadIdx.x;
     tridiagonalise(C, m, sh);
     bisect_prepare(m, sh);
@@ -991,7 +994,7 @@ __device__ double range_sum(double* __restrict__ C, int m, double xl, double xh,
 // point of the bracket, which shrinks 33-fold; float32 counts first, then the
 // widened bracket is checked and refined with float64 counts.  Result in
 // sh.red[0] (read after a barrier).
-__device__ void max_eig_warp(int n, Shared& sh) {
+__device__ __noinline__ void max_eig_warp(int n, Shared& sh) {
     const int lane = threadIdx.x & 31;
     const float* d32 = reinterpret_cast<const float*>(sh.rs);
     const float* e32 = d32 + n;
@@ -1034,7 +1037,7 @@ __device__ void max_eig_warp(int n, Shared& sh) {
 // of 32 rows, each thread a 2 x 2 block of outputs with independent
 // accumulators.  With `upper` only tiles on or above the diagonal are formed and
 // every value is also stored at (q, p) (A^T B symmetric, e.g. Z^T T Z).
-__device__ void gemm_tn(const double* __restrict__ Am, int lda, const double* __restrict__ Bm, int ldb, int K,
+__device__ __noinline__ void gemm_tn(const double* __restrict__ Am, int lda, const double* __restrict__ Bm, int ldb, int K,
                         int P, int Q, double* __restrict__ C, int ldc, bool upper, Shared& sh) {
     double* ta = sh.gt;            // [32 k][33]
     double* tb = sh.gt + 32 * 33;  // [32 k][33]
@@ -1106,7 +1109,7 @@ __device__ void gemm_tn(const double* __restrict__ Am, int lda, const double* __
 // vector is not finite, its residual exceeds 1e3 n eps ||T||, or two
 // neighbouring vectors are not orthogonal to 1e-6 (nearly equal eigenvalues):
 // the caller then takes the QL route.
-__device__ void twisted_vectors(int n, int r, double* __restrict__ Z, double* __restrict__ Dp,
+__device__ __noinline__ void twisted_vectors(int n, int r, double* __restrict__ Z, double* __restrict__ Dp,
                                 double* __restrict__ Dm, int ldz, Shared& sh) {
     const int tid = threadIdx.x;
     if (tid == 0) {
@@ -1242,7 +1245,7 @@ __device__ void back_transform_cols(const double* __restrict__ A, int n, double*
 // Householder factor left by tridiagonalise (vector k in row k of A from column
 // k+1, scalar sh.beta[k]): the eigenvectors of T become those of the matrix it
 // was reduced from.  One thread per column.
-__device__ void back_transform(const double* __restrict__ A, int n, double* __restrict__ Z, int ldz, int r,
+__device__ __noinline__ void back_transform(const double* __restrict__ A, int n, double* __restrict__ Z, int ldz, int r,
                                const Shared& sh) {
     const int nw = (int)(blockDim.x >> 5);
     if (r <= nw) {
@@ -1297,7 +1300,7 @@ __device__ void back_transform(const double* __restrict__ A, int n, double* __re
 // its scalar, so that H_{d-1} ... H_0 Q is upper triangular; the span of Q is
 // that of the first d columns of H_0 ... H_{d-1}, its orthogonal complement that
 // of the others.
-__device__ void householder_qr_cols(double* __restrict__ Q, int ldq, int n, int d, Shared& sh) {
+__device__ __noinline__ void householder_qr_cols(double* __restrict__ Q, int ldq, int n, int d, Shared& sh) {
     const int tid = threadIdx.x;
     for (int j = 0; j < d; ++j) {
         double f = 0.0;
@@ -1335,7 +1338,7 @@ __device__ void householder_qr_cols(double* __restrict__ Q, int ldq, int n, int 
 // reflection j reaches the trailing block during the pass (sym_pass) that forms the
 // product K u_{j+1} of the next one: one read and one write of the lower triangle per
 // reflection and matrix.  Uses sh.v, sh.p, sh.rc, sh.rs, sh.d, sh.off as vectors.
-__device__ void reflect_all(double* __restrict__ K1, double* __restrict__ K2, int n, const double* __restrict__ Q,
+__device__ __noinline__ void reflect_all(double* __restrict__ K1, double* __restrict__ K2, int n, const double* __restrict__ Q,
                             int ldq, int d, Shared& sh) {
     const int tid = threadIdx.x, nthr = (int)blockDim.x;
     double* uc = sh.v;   // this reflection's u
