@@ -469,6 +469,56 @@ __global__ void moments_tc_seg_kernel(const double* __restrict__ ge, const doubl
     }
 }
 
+// The same sums and the moments of a step in one launch, for batches of small matrices: one
+// thread an element pair (i, j), (j, i), the chains of sum_tc_kernel one after the other (an
+// empty chain adds nothing).
+__device__ __forceinline__ double chain_sum(const float* __restrict__ p, size_t nn, size_t e, int k0, int k1) {
+    double s = 0.0;
+    const int k8 = min(k1, k0 + 8);
+#pragma unroll 1
+    for (int k = k0; k < k8; ++k) {
+        Sum32 a;
+        sum_slabs(a, p, nn, e, k, k1);
+        s += a.value();
+    }
+    return s;
+}
+
+__global__ void __launch_bounds__(256)
+step_tc_seg_kernel(const float* __restrict__ pe, const float* __restrict__ po, const int* __restrict__ seg, int B,
+                   int n_tot, double* __restrict__ X, size_t xstride, int step) {
+    const size_t nn = (size_t)n_tot * n_tot;
+    const int b = blockIdx.y;
+    const int e0 = seg[b], e1 = seg[b + 1], o0 = seg[B + 1 + b], o1 = seg[B + 2 + b];
+    double* Xb = X + (size_t)b * xstride;
+    const unsigned npair = (unsigned)n_tot * (n_tot + 1) / 2;
+    for (unsigned u = blockIdx.x * blockDim.x + threadIdx.x; u < npair; u += gridDim.x * blockDim.x) {
+        // u -> (i, j), i <= j: row i of the upper triangle starts at i n_tot - i (i - 1) / 2
+        const unsigned m = npair - 1 - u;  // counted from the end: t (t + 1) / 2 <= m
+        unsigned t = (unsigned)((sqrtf(8.f * (float)m + 1.f) - 1.f) * 0.5f);
+        while (t * (t + 1) / 2 > m) --t;
+        while ((t + 1) * (t + 2) / 2 <= m) ++t;
+        const unsigned i = n_tot - 1 - t, j = n_tot - 1 - (m - t * (t + 1) / 2);
+        const size_t e = (size_t)i * n_tot + j, tr = (size_t)j * n_tot + i;
+        const double gs = chain_sum(pe, nn, e, e0, e1);
+        if (step < 0) {
+            Xb[e] = Xb[tr] = gs;
+            continue;
+        }
+        const double gc = 0.5 * (chain_sum(po, nn, e, o0, o1) + chain_sum(po, nn, tr, o0, o1));
+        const double x0 = Xb[e];
+        if (step == 0) {
+            Xb[nn + e] = Xb[nn + tr] = gc;
+            Xb[2 * nn + e] = Xb[2 * nn + tr] = 2.0 * gs - x0;
+        } else {
+            double* odd = Xb + (size_t)(2 * step + 1) * nn;
+            double* even = Xb + (size_t)(2 * step + 2) * nn;
+            odd[e] = odd[tr] = 2.0 * gc - Xb[nn + e];
+            even[e] = even[tr] = 2.0 * gs - x0;
+        }
+    }
+}
+
 // Fused-step partials (fused_tc.cu): slab s holds accumulator rows 0..127 for
 // s < nA and rows 128.. for s >= nA, so element (i, j) sums the slabs of its
 // row range, in the fixed order of sum_tc_kernel.  blockIdx.y selects the step.
@@ -613,6 +663,17 @@ cudaError_t launch_reduce_tc_batch(const float* ring, int n_e, int n_o, int n_to
 cudaError_t launch_reduce_tc_seg(const float* part, int n_e, int n_tot, int B, const int* seg, double* ge,
                                  double* go, double* X, size_t xstride, int step, cudaStream_t s) {
     const int64_t nn = (int64_t)n_tot * n_tot;
+    // Few slabs a matrix and many matrices: a thread an element.  The eight warps an element of
+    // the other path spend the float64 pipe on converting and adding zeros there (1100 matrices
+    // of one slab, n_tot = 32: 125 us and 14 us for the moments, against 24 us); with more
+    // slabs than warps they share the loads.
+    if (n_e <= (int64_t)4 * B) {
+        int64_t pb = (nn / 2 + n_tot + 255) / 256;
+        if (pb > 64) pb = 64;
+        step_tc_seg_kernel<<<dim3((unsigned)pb, (unsigned)B), 256, 0, s>>>(part, part + (size_t)n_e * nn, seg, B, n_tot,
+                                                                         X, xstride, step);
+        return cudaGetLastError();
+    }
     int64_t sb = (nn + 31) / 32;
     if (sb > 64) sb = 64;
     dim3 sg((unsigned)sb, (unsigned)B);
