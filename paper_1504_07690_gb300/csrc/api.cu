@@ -539,7 +539,7 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
             // (no use where every point runs the serial QL chains, or a warp-size kernel first)
             if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P)) &&
                 !solve_uses_small(n_t, nv, nvh, (P.p.options & SSM_OPT_PINV) != 0)) {
-                const int64_t slots = solve_slots(nv, hybrid_routes(P));
+                const int64_t slots = solve_slots(nv, hybrid_routes(P), n_t);
                 if (slots >= n_t) {
                     if ((size_t)slots > h->cap_perm) {
                         dev_free(h->d_perm);

@@ -366,7 +366,7 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
                          bool pinv = false, bool hyb = false, int32_t* pend = nullptr);
 // Resident solver CTAs on the device (SMs x CTAs per SM; 0 if not available): the
 // slots of one wave, the length of a schedule.
-int64_t solve_slots(int n_v, bool hyb);
+int64_t solve_slots(int n_v, bool hyb, int64_t n_t);
 // Whether a launch_solve with room in `pend` runs the warp-per-point kernel first.
 bool solve_uses_small(int64_t n_t, int n_v, int n_vh, bool pinv);
 // Schedule (perm, solve_slots(n_v) entries) of the next solve launch over n_t points

@@ -12,6 +12,17 @@ namespace {
 // per SM).
 int solve_threads(int n_v) { return n_v <= 128 ? 128 : NT; }
 
+// ... but a launch of few points lasts as long as its slowest ones, and a float64 fma holds
+// its warp for 65 cycles of which the pipe is busy 16: eight warps a point, for points with
+// hybrid columns up to four an SM (400 points of n_v = 128, n_vh = 128: 12.4 ms against 18.3;
+// 600 of n_v = 100: 7.5 against 8.6, 900: no gain), without up to two (20 points of n_v = 100:
+// 5.1 against 6.4; where every point keeps a part of its directions 300 take 7.4 against 7.8,
+// 450 9.3 against 9.1).  The step-by-step route of float64 plans keeps its sums' order.
+int solve_threads(int n_v, int n_vh, bool hyb, int64_t n_t) {
+    const int per_sm = hyb ? (n_v > 32 ? 4 : 0) : (n_vh == 0 && n_v > 64 ? 2 : 0);
+    return n_t <= (int64_t)per_sm * device_sms() ? NT : solve_threads(n_v);
+}
+
 // CTAs with a private workspace: 4 x (256 / threads) per SM to overlap the
 // serial QL chains, fewer when their workspaces would exceed 2 GiB in total.
 int workspace_ctas(int n_v, bool hyb) {
@@ -100,7 +111,7 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
     if (e != cudaSuccess) return e;
     int64_t grid = workspace_ctas(n_v, hyb), n_slot = n_t;
     if (perm) {
-        n_slot = solve_slots(n_v, hyb);
+        n_slot = solve_slots(n_v, hyb, n_t);
         if (n_slot < n_t || n_slot > grid) return cudaErrorInvalidValue;
     }
     if (grid > n_slot) grid = n_slot;
@@ -113,9 +124,9 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
         n_dev = pend;
         perm = pend + 1;
     }
-    kernel<<<(int)grid, solve_threads(n_v), smem, s>>>(Kfull, KZ, n_t, n_v, n_vh, tau, xlo, xhi, mu, ldmu, K,
-                                                   floor_scale, (double*)work, dos, rank, flag, floor_pt, perm,
-                                                   n_slot, pinv, n_dev);
+    kernel<<<(int)grid, solve_threads(n_v, n_vh, hyb, n_t), smem, s>>>(Kfull, KZ, n_t, n_v, n_vh, tau, xlo, xhi, mu,
+                                                                       ldmu, K, floor_scale, (double*)work, dos, rank,
+                                                                       flag, floor_pt, perm, n_slot, pinv, n_dev);
     return cudaGetLastError();
 }
 
@@ -127,14 +138,14 @@ bool solve_uses_small(int64_t n_t, int n_v, int n_vh, bool pinv) {
     return n_v <= SOLVE_SMALL_N && n_vh == 0 && !pinv && n_t >= (int64_t)8 * device_sms();
 }
 
-int64_t solve_slots(int n_v, bool hyb) {
+int64_t solve_slots(int n_v, bool hyb, int64_t n_t) {
     int dev = 0, sms = 0, k = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t smem = solve_smem(n_v);
     const SolveKernel kernel = hyb ? solve_kernel_hyb() : solve_kernel<false>;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, kernel, solve_threads(n_v), smem) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, kernel, solve_threads(n_v, hyb ? 1 : 0, hyb, n_t), smem) != cudaSuccess)
         return 0;
     const int64_t slots = (int64_t)sms * k;
     return slots <= workspace_ctas(n_v, hyb) ? slots : 0;
@@ -145,7 +156,7 @@ cudaError_t launch_solve_schedule(const int32_t* rank_prev, int64_t n_t, int n_v
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t slots = solve_slots(n_v, hyb);
+    const int64_t slots = solve_slots(n_v, hyb, n_t);
     if (slots < n_t || slots <= 0) return cudaErrorInvalidValue;
     const size_t smem = (size_t)(slots + n_t) * sizeof(int32_t);
     if (smem > 48 * 1024) return cudaErrorInvalidValue;
