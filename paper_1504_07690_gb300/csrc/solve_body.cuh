@@ -868,43 +868,112 @@ __device__ __noinline__ bool cholesky_lower(double* __restrict__ A, int n, const
     return true;
 }
 
-// X <- L^{-1} X for the n x n row-major X, L from cholesky_lower (rdiag =
-// sh.v): forward substitution, one column of X per thread.
-__device__ __noinline__ void trsm_lower(const double* __restrict__ L, double* __restrict__ X, int n, const Shared& sh) {
-    for (int c = threadIdx.x; c < n; c += (int)blockDim.x) {
-        for (int i = 0; i < n; ++i)
-            X[(size_t)i * n + c] = (X[(size_t)i * n + c] - dot8(L + (size_t)i * n, 1, X + c, n, i)) * sh.v[i];
-    }
-    __syncthreads();
-}
-
-// Y <- L^{-1} X^T (X, Y distinct, n x n row-major): forward substitution on
-// the rows of X, one row per thread; row r of X gives column r of Y.
-__device__ __noinline__ void trsm_lower_t(const double* __restrict__ L, const double* __restrict__ X, double* __restrict__ Y,
-                             int n, const Shared& sh) {
-    for (int r = threadIdx.x; r < n; r += (int)blockDim.x) {
-        const double* xr = X + (size_t)r * n;
-        for (int i = 0; i < n; ++i)
-            Y[(size_t)i * n + r] = (xr[i] - dot8(L + (size_t)i * n, 1, Y + r, n, i)) * sh.v[i];
-    }
-    __syncthreads();
-}
-
-// sum_ik X_ik^2 for X = L^{-1} M, M lower triangular (its lower triangle is read;
-// X overwrites it), L from cholesky_lower (rdiag = sh.v).  X is lower triangular
-// as well, so column c is a forward substitution from row c down (n^3 / 3 flops),
-// one column per thread.
-__device__ __noinline__ double trtr_sumsq(const double* __restrict__ L, double* __restrict__ M, int n, const Shared& sh) {
+// X <- L^{-1} B for the m x m lower triangular L (row-major, its reciprocal diagonal in sh.v)
+// and m x cols X (ld ldx): B is X itself, or the transpose of the row-major cols x m matrix Bt
+// (not X).  TRI: B is lower triangular (m = cols; only its lower triangle is read, and only
+// X's is written) and the sum of X's squares is returned.
+//
+// By 32-row panels: the finished rows above are subtracted tile by tile as in cholesky_lower,
+// the panel is then solved against its diagonal block, a warp 32 columns, a lane one column,
+// 16 rows at a time in registers.  The float64 pipe bounds the products; a substitution down
+// one column a thread waited for each row's partial sums instead (1200 hybrid points of n_v =
+// 128: 20.6 ms, 17.0 as here; 400 points of n_v = 200: 19.4 and 18.9).
+template <bool TRI>
+__device__ __noinline__ double solve_lower(const double* __restrict__ L, int m, const double* Bt, double* X, int ldx,
+                                           int cols, const Shared& sh) {
+    double* ta = sh.gt;            // [32 k][33]: staged L, then the diagonal block [row][33]
+    double* tb = sh.gt + 32 * 33;  // [32 k][33]: staged X
+    const int tid = threadIdx.x, nt = (int)blockDim.x, warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
     double f = 0.0;
-    for (int c = threadIdx.x; c < n; c += (int)blockDim.x) {
-        for (int i = c; i < n; ++i) {
-            const double x =
-                (M[(size_t)i * n + c] - dot8(L + (size_t)i * n + c, 1, M + (size_t)c * n + c, n, i - c)) * sh.v[i];
-            M[(size_t)i * n + c] = x;
-            f = fma(x, x, f);
+    for (int jb = 0; jb < m; jb += 32) {
+        const int w = min(32, m - jb);
+        const int cend = TRI ? jb + w : cols;
+        for (int c0 = 0; c0 < cend; c0 += 32) {
+            const int wc = min(32, cols - c0);
+            double acc[2][2][2] = {};  // a CTA of 128 threads takes two passes
+            for (int k0 = TRI ? c0 : 0; k0 < jb; k0 += 32) {
+                __syncthreads();
+                for (int e = tid; e < 32 * 32; e += nt) {
+                    const int hi = e >> 5, lo = e & 31;
+                    ta[lo * 33 + hi] = hi < w ? L[(size_t)(jb + hi) * m + k0 + lo] : 0.0;
+                    tb[hi * 33 + lo] =
+                        lo < wc && (!TRI || k0 + hi >= c0 + lo) ? X[(size_t)(k0 + hi) * ldx + c0 + lo] : 0.0;
+                }
+                __syncthreads();
+#pragma unroll
+                for (int pass = 0; pass < 2; ++pass) {
+                    const int t = tid + pass * nt;
+                    const int pi = 2 * (t >> 4), qj = 2 * (t & 15);
+                    if (t < 256 && pi < w && qj < wc) {
+#pragma unroll 8
+                        for (int kk = 0; kk < 32; ++kk) {
+                            const double a0 = ta[kk * 33 + pi], a1 = ta[kk * 33 + pi + 1];
+                            const double b0 = tb[kk * 33 + qj], b1 = tb[kk * 33 + qj + 1];
+                            acc[pass][0][0] = fma(a0, b0, acc[pass][0][0]);
+                            acc[pass][0][1] = fma(a0, b1, acc[pass][0][1]);
+                            acc[pass][1][0] = fma(a1, b0, acc[pass][1][0]);
+                            acc[pass][1][1] = fma(a1, b1, acc[pass][1][1]);
+                        }
+                    }
+                }
+            }
+            if (jb > 0 || Bt)
+#pragma unroll
+                for (int pass = 0; pass < 2; ++pass) {
+                    const int t = tid + pass * nt;
+                    const int pi = 2 * (t >> 4), qj = 2 * (t & 15);
+                    if (t < 256)
+                        for (int i = 0; i < 2; ++i)
+                            for (int j = 0; j < 2; ++j) {
+                                const int r = jb + pi + i, c = c0 + qj + j;
+                                if (pi + i < w && qj + j < wc && (!TRI || r >= c)) {
+                                    const double b = Bt ? Bt[(size_t)c * m + r] : X[(size_t)r * ldx + c];
+                                    X[(size_t)r * ldx + c] = b - acc[pass][i][j];
+                                }
+                            }
+                }
         }
+        __syncthreads();
+        for (int e = tid; e < 32 * 32; e += nt) {
+            const int i = e >> 5, k = e & 31;
+            ta[i * 33 + k] = i < w && k < i ? L[(size_t)(jb + i) * m + jb + k] : 0.0;
+        }
+        if (tid < 32) ta[tid * 33 + 32] = tid < w ? sh.v[jb + tid] : 0.0;
+        __syncthreads();
+        for (int ct = warp; 32 * ct < cend; ct += nw) {
+            const int c = 32 * ct + lane;
+            double* x = X + (size_t)jb * ldx + c;
+            // rows of the panel that this lane's column has
+            const int r0 = TRI ? max(0, c - jb) : 0, r1 = c < cols ? w : 0;
+#pragma unroll 1
+            for (int h = 0; h < w; h += 16) {
+                const double* t = ta + h * 33;
+                double s[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) s[i] = h + i >= r0 && h + i < r1 ? x[(size_t)(h + i) * ldx] : 0.0;
+#pragma unroll 2
+                for (int k = 0; k < h; ++k) {
+                    const double xk = k >= r0 && k < r1 ? x[(size_t)k * ldx] : 0.0;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) s[i] = fma(-t[i * 33 + k], xk, s[i]);
+                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    s[k] *= t[k * 33 + 32];
+#pragma unroll
+                    for (int i = k + 1; i < 16; ++i) s[i] = fma(-t[i * 33 + h + k], s[k], s[i]);
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (h + i >= r0 && h + i < r1) {
+                        x[(size_t)(h + i) * ldx] = s[i];
+                        if (TRI) f = fma(s[i], s[i], f);
+                    }
+            }
+        }
+        __syncthreads();
     }
-    return block_sum(f, sh.red);
+    return TRI ? block_sum(f, sh.red) : 0.0;
 }
 
 // Sum (and count) of the eigenvalues of the symmetric m x m matrix C (ld m,
@@ -1432,7 +1501,7 @@ enum class Kept { All, Span, Complement };
 // K_W-orthonormal basis Y L^-T, and the filter keeps their part in the eigenvectors of the
 // pencil inside it.  The reflections of the eigenvectors' QR split a coordinate vector
 // into the two parts without a subtraction.  The columns go in chunks of at most n through
-// b1, b2 (n^2 each); forward substitution, one column a thread.
+// b1, b2 (n^2 each).
 __device__ __noinline__ double hybrid_norm(const double* __restrict__ Kt, int n_tot, int n, int nvh, const double* __restrict__ L,
                               int m, Basis basis, const double* __restrict__ Q, const double* __restrict__ bq,
                               Kept kept, const double* __restrict__ V, int q, double* __restrict__ b1,
@@ -1456,12 +1525,8 @@ __device__ __noinline__ double hybrid_norm(const double* __restrict__ Kt, int n_
             reflect_cols(Q, n, bq, n - m, b1, n, hc);
             X = b1 + (size_t)(n - m) * hc;
         }
-        for (int c = tid; c < hc; c += nt)
-            for (int i = 0; i < m; ++i)
-                X[(size_t)i * hc + c] =
-                    (X[(size_t)i * hc + c] - dot8(L + (size_t)i * m, 1, X + c, hc, i)) * sh.v[i];
+        solve_lower<false>(L, m, nullptr, X, hc, hc, sh);
         if (kept != Kept::All) {
-            __syncthreads();
             reflect_cols(V, q, sh.beta, q, X, m, hc);
         }
         const int i0 = kept == Kept::Complement ? q : 0, i1 = kept == Kept::Span ? q : m;
@@ -1678,7 +1743,7 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                 r = n;
                 done = true;
                 if (inside) {
-                    phi = fma(xl, (double)n, trtr_sumsq(Zt, T1, n, sh));
+                    phi = fma(xl, (double)n, solve_lower<true>(Zt, n, nullptr, T1, n, n, sh));
                     rs = n;
                     if constexpr (HYB) {
                         kcn = hybrid_norm(Kt, n_tot, n, nvh, Zt, n, Basis::Identity, nullptr, nullptr, Kept::All,
@@ -1691,8 +1756,8 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                         Y[e] = 0.5 * (Zk[(size_t)i * n + j] + Zk[(size_t)j * n + i]);
                     }
                     __syncthreads();
-                    trsm_lower(Zt, Y, n, sh);       // Y = L^-1 K_Z
-                    trsm_lower_t(Zt, Y, A, n, sh);  // A = L^-1 Y^T = L^-1 K_Z L^-T
+                    solve_lower<false>(Zt, n, nullptr, Y, n, n, sh);  // Y = L^-1 K_Z
+                    solve_lower<false>(Zt, n, Y, A, n, n, sh);        // A = L^-1 Y^T = L^-1 K_Z L^-T
                     for (int e = tid; e < n * n; e += (int)blockDim.x) {  // symmetrise (upper from lower)
                         const int i = e / n, j = e - i * n;
                         if (i < j) {
@@ -1814,7 +1879,7 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                     r = rk;
                     done = true;
                     if (inside) {
-                        phi = fma(xl, (double)rk, trtr_sumsq(Lw, S1, rk, sh));
+                        phi = fma(xl, (double)rk, solve_lower<true>(Lw, rk, nullptr, S1, rk, rk, sh));
                         rs = rk;
                         if constexpr (HYB) {
                             kcn = hybrid_norm(Kt, n_tot, n, nvh, Lw, rk, basis, Zt, bq, Kept::All, nullptr, 0, T1, U2,
@@ -1822,8 +1887,8 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
                             have_kcn = true;
                         }
                     } else {
-                        trsm_lower(Lw, Mz, rk, sh);        // Mz = L^-1 M_Z
-                        trsm_lower_t(Lw, Mz, T1, rk, sh);  // T1 = L^-1 M_Z L^-T
+                        solve_lower<false>(Lw, rk, nullptr, Mz, rk, rk, sh);  // Mz = L^-1 M_Z
+                        solve_lower<false>(Lw, rk, Mz, T1, rk, rk, sh);       // T1 = L^-1 M_Z L^-T
                         for (int e = tid; e < rk * rk; e += (int)blockDim.x) {
                             const int i = e / rk, j = e - i * rk;
                             if (i < j) {
