@@ -32,8 +32,8 @@
 //
 // TMEM: Ge uses ntp (+ ntp-128) columns, Go ntp (+ ntp) columns, ntp = n_tot
 // rounded up to 16, n_tot <= 256; a CTA allocates all 512 columns and its
-// shared-memory footprint keeps it alone on its SM (two CTAs with half of each share an SM
-// where slabs are small and blocks narrow).  Every wait is bounded:
+// shared-memory footprint keeps it alone on its SM (two or four CTAs with their parts of
+// each share an SM where slabs are small and blocks narrow).  Every wait is bounded:
 // on expiry the CTA sets bit 2 of the status word, waits once more (bounded)
 // for its MMAs, frees TMEM and returns.
 #include <cuda_bf16.h>
@@ -88,7 +88,7 @@ struct TcArgs {
     uint32_t smem_bytes, tmem_cols;  // of a CTA
 };
 
-__global__ void __launch_bounds__(NTHREADS, 2) gram_tc_kernel(TcArgs P) {
+__global__ void __launch_bounds__(NTHREADS, 4) gram_tc_kernel(TcArgs P) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t full[STAGES], empty[STAGES], done;
     __shared__ uint32_t tmem_slot;
@@ -618,12 +618,16 @@ cudaError_t launch_gram_tc(const uint8_t* PX, const uint8_t* PY, int n_tot, int6
     a.slabs = slabs;
     a.both = both && PY;
     // Narrow blocks in small slabs (batched plans): a CTA's life is its latencies, one after
-    // the other (allocation, first copies, MMA chain, epilogue), so two share an SM, each
-    // with half of the tensor memory and of the shared memory (1100 slabs of about 16 panels,
-    // n_tot = 32: the recurrence graph of 50 steps 10.1 -> 8.7 ms, n_tot = 16: 6.6 -> 5.4 ms).
-    const bool half = slabs && (n_tot + 15) / 16 * 16 <= 64 && n_e >= 2 * device_sms();
-    a.smem_bytes = half ? SMEM_BYTES / 2 : SMEM_BYTES;
-    a.tmem_cols = half ? TMEM_COLS / 2 : TMEM_COLS;
+    // the other (allocation, first copies, MMA chain, epilogue), so four share an SM (n_tot <=
+    // 32; two up to 64, whose ring would be one stage), each with its part of the tensor memory
+    // and of the shared memory.  1100 slabs of about 16 panels, the recurrence graph of 50
+    // steps: n_tot = 32 10.1 ms with one, 8.8 with two, 8.1 with four; n_tot = 16 6.6, 5.3 and
+    // 4.8; n_tot = 56 14.8 with two, 15.2 with four.
+    const int ntp = (n_tot + 15) / 16 * 16, sms = device_sms();
+    int share = 1;
+    if (slabs && ntp <= 64 && n_e >= 2 * sms) share = ntp <= 32 && n_e >= 4 * sms ? 4 : 2;
+    a.smem_bytes = SMEM_BYTES / share;
+    a.tmem_cols = TMEM_COLS / share;
     gram_tc_kernel<<<a.both ? a.n_e : a.n_e + a.n_o, NTHREADS, a.smem_bytes, s>>>(a);
     return cudaGetLastError();
 }
