@@ -2112,24 +2112,25 @@ ssm_status trace_prepare(ssm_plan_s* h, double (*f)(double, void*), void* ctx, i
     const double fend = 0.5 * (f0 + f1);
     ssm_status s = ensure_points(h, n_t);
     if (s != SSM_OK) return s;
-    if ((size_t)(10 * n_t + 2) > h->cap_tr) {
+    if ((size_t)(12 * n_t + 2) > h->cap_tr) {
         dev_free(h->d_tr);
         h->d_tr = nullptr;
         h->cap_tr = 0;
-        CUDA_OR_FAIL(h, dev_alloc(&h->d_tr, 10 * n_t + 2));
-        h->cap_tr = 10 * n_t + 2;
+        CUDA_OR_FAIL(h, dev_alloc(&h->d_tr, 12 * n_t + 2));
+        h->cap_tr = 12 * n_t + 2;
     }
     double* d_tt = h->d_tr;
     double* d_fx = d_tt + 2 * n_t;
     double* d_h = d_fx + n_t;
     double* d_ft = d_h + n_t;
     double* d_work = d_ft + n_t;   // 5 n_t
+    double* d_tw = h->d_tr + 10 * n_t + 2;
     CUDA_OR_FAIL(h, cudaMemcpyAsync(d_tt, host.data(), 3 * n_t * sizeof(double), cudaMemcpyHostToDevice, P.stream));
     {
         Scope sc(h, PH_TRACE);
         CUDA_OR_FAIL(h, launch_trace_h(d_tt, d_fx, n_t, fend, a, sigma_tilde, d_h, P.stream));
-        CUDA_OR_FAIL(h, launch_deconvolve(d_h, n_t, dx, sigma, DECONV_CUTOFF, d_work, d_ft, P.stream));
-        P.stats.launches += 4;
+        CUDA_OR_FAIL(h, launch_deconvolve(d_h, n_t, dx, sigma, DECONV_CUTOFF, d_work, d_tw, d_ft, P.stream));
+        P.stats.launches += 6;
     }
     *dx_out = dx;
     return SSM_OK;

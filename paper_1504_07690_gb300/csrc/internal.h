@@ -396,7 +396,7 @@ cudaError_t launch_kpm_adjoint(const double* mu, int ldmu, int64_t n_t, int L, c
 cudaError_t launch_trace_h(const double* tt, const double* fx, int64_t n_t, double fend, double a,
                            double sigma_tilde, double* h, cudaStream_t s);
 cudaError_t launch_deconvolve(const double* h, int64_t n_t, double dx, double sigma, double cutoff,
-                              double* work, double* ftilde, cudaStream_t s);
+                              double* work, double* tw, double* ftilde, cudaStream_t s);
 cudaError_t launch_trace_dot(const double* ftilde, const double* dos, int64_t n_t, double scale,
                              double* out, cudaStream_t s);
 
