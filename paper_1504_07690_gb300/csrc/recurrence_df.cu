@@ -33,8 +33,8 @@ struct F2 {
 };
 
 // Two columns' float pairs, each operation on both at once (f32x2 instructions, rounded as
-// the scalar ones): the step is bound by instruction issue (65 to 70 % active at 139 us a
-// step of 65536 x 200), and this halves the arithmetic.
+// the scalar ones): the step was bound by instruction issue (65 to 70 % active at 139 us a
+// step of 65536 x 200), and this halves the arithmetic (101 us).
 struct P2 {
     pair32 h, l;
 };
