@@ -316,6 +316,117 @@ __device__ void tridiagonalise(double* __restrict__ A, int n, Shared& sh) {
     __syncthreads();
 }
 
+// The same reduction for the factored routes, on the whole symmetric matrix (both triangles are
+// read and kept): a thread owns a column of the trailing matrix and walks down its rows, so the
+// rank-2 update and the product p = A22 v need no staging, no barrier and no reduction but
+// that of the row groups (as many as the CTA's threads allow).  3 fma an element of the square
+// against 4 an element of the triangle, whose tiles are padded and take two phases (a point of
+// n = 200 that keeps three directions, alone on its SM: 7.9 ms by tiles, 7.3 so; 20 points of
+// n = 100 that keep a part: 5.0 and 4.7).  Layout of the reflectors as tridiagonalise;
+// blockDim.x >= n.
+__device__ __noinline__ void tridiagonalise_square(double* __restrict__ A, int n, Shared& sh) {
+    const int tid = threadIdx.x, nthr = (int)blockDim.x;
+    double* vc = sh.v;
+    double* wc = sh.p;
+    double* vq = sh.rc;  // the pending update (previous step): v
+    double* wq = sh.rs;  //                                     w
+    double* part = sh.gt;
+    bool pending = false;
+    for (int k = 0; k + 2 < n; ++k) {
+        const int L = n - k - 1;
+        double* T = A + (size_t)(k + 1) * n + k + 1;
+        const double x = tid < L ? A[(size_t)k * n + k + 1 + tid] : 0.0;  // row k right of the diagonal
+        const double nrm2 = block_sum(x * x, sh.red);
+        const double x0 = A[(size_t)k * n + k + 1];
+        double beta = 0.0, alpha = x0, v = 0.0;
+        if (nrm2 - x0 * x0 > 0.0) {
+            alpha = -copysign(sqrt(nrm2), x0);
+            const double v0 = x0 - alpha;
+            beta = 2.0 / (nrm2 - x0 * x0 + v0 * v0);
+            v = tid == 0 ? v0 : x;
+            if (tid < L) vc[tid] = v;
+        }
+        if (tid == 0) {
+            sh.d[k] = A[(size_t)k * n + k];
+            sh.off[k] = alpha;
+            sh.beta[k] = beta;
+        }
+        __syncthreads();
+        const bool sums = beta != 0.0;
+        if (sums && tid < L) A[(size_t)k * n + k + 1 + tid] = v;
+        const int Lp = (L + 31) & ~31, G = nthr / Lp, g = tid / Lp, i = tid - g * Lp;
+        const int per = (L + G - 1) / G;
+        if ((sums || pending) && g < G && i < L) {
+            const double vi = pending ? vq[i + 1] : 0.0, wi = pending ? wq[i + 1] : 0.0;
+            const int j1 = min(L, (g + 1) * per);
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            int j = g * per;
+            for (; j + 8 <= j1; j += 8) {
+                double a[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) a[u] = T[(size_t)(j + u) * n + i];
+                if (pending) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        a[u] = fma(-vq[j + u + 1], wi, fma(-wq[j + u + 1], vi, a[u]));
+                        T[(size_t)(j + u) * n + i] = a[u];
+                    }
+                }
+                if (sums) {
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) s[u & 3] = fma(a[u], vc[j + u], s[u & 3]);
+                }
+            }
+            for (; j < j1; ++j) {
+                double a = T[(size_t)j * n + i];
+                if (pending) {
+                    a = fma(-vq[j + 1], wi, fma(-wq[j + 1], vi, a));
+                    T[(size_t)j * n + i] = a;
+                }
+                if (sums) s[0] = fma(a, vc[j], s[0]);
+            }
+            part[g * Lp + i] = (s[0] + s[1]) + (s[2] + s[3]);
+        }
+        if (sums) {
+            __syncthreads();
+            double w = 0.0;
+            if (tid < L) {
+                for (int q = 0; q < G; ++q) w += part[q * Lp + tid];
+                w *= beta;
+            }
+            const double K = 0.5 * beta * block_sum(w * v, sh.red);
+            w -= K * v;  // p becomes w
+            if (tid < L) wc[tid] = w;
+            __syncthreads();
+            // row k+1 (with its diagonal) takes this step's update now
+            if (tid < L) T[tid] = fma(-v, wc[0], fma(-w, vc[0], T[tid]));
+        }
+        pending = sums;
+        double* t = vc;
+        vc = vq;
+        vq = t;
+        t = wc;
+        wc = wq;
+        wq = t;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        if (pending) {  // the last update on the last diagonal element (frame of step n-3)
+            double* e = A + (size_t)(n - 1) * n + n - 1;
+            *e = fma(-vq[1], wq[1], fma(-wq[1], vq[1], *e));
+        }
+        if (n >= 2) {
+            sh.d[n - 2] = A[(size_t)(n - 2) * n + n - 2];
+            sh.off[n - 2] = A[(size_t)(n - 2) * n + n - 1];
+            sh.beta[n - 2] = 0.0;
+        }
+        sh.d[n - 1] = A[(size_t)(n - 1) * n + n - 1];
+        sh.off[n - 1] = 0.0;
+        if (n >= 2) sh.beta[n - 1] = 0.0;
+    }
+    __syncthreads();
+}
+
 // Zt = H^T (rows of Zt are the columns of H = H_0 H_1 ... H_{n-3}), from the
 // vectors left in A by tridiagonalise.  Backward accumulation on H, written
 // transposed: column j of H ends up in row j of Zt.
@@ -1022,7 +1133,7 @@ __device__ __noinline__ double solve_lower(const double* __restrict__ L, int m, 
 // the eigenvalues inside.
 __device__ __noinline__ double range_sum(double* __restrict__ C, int m, double xl, double xh, Shared& sh, int* count) {
     const int tid = threadIdx.x;
-    tridiagonalise(C, m, sh);
+    tridiagonalise_square(C, m, sh);
     bisect_prepare(m, sh);
     if (tid == 0) {
         sh.misc[0] = max(0, sturm_below(sh.d, sh.p, m, xl) - 1);
@@ -1731,7 +1842,10 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
             }
         }
         if (!full && !empty) {
-            tridiagonalise(A, n, sh);
+            if (routes)
+                tridiagonalise_square(A, n, sh);
+            else
+                tridiagonalise(A, n, sh);
             bisect_prepare(n, sh);
             if (tid < 32) max_eig_warp(n, sh);
             __syncthreads();
