@@ -322,8 +322,8 @@ __device__ void tridiagonalise(double* __restrict__ A, int n, Shared& sh) {
 // that of the row groups (as many as the CTA's threads allow).  3 fma an element of the square
 // against 4 an element of the triangle, whose tiles are padded and take two phases (a point of
 // n = 200 that keeps three directions, alone on its SM: 7.9 ms by tiles, 7.3 so; 20 points of
-// n = 100 that keep a part: 5.0 and 4.7).  Layout of the reflectors as tridiagonalise;
-// blockDim.x >= n.
+// n = 100 that keep a part: 5.0 and 4.7).  Layout of the reflectors as tridiagonalise; the
+// trailing block needs a thread a column: n - 1 <= blockDim.x (tridiagonalise_route).
 __device__ __noinline__ void tridiagonalise_square(double* __restrict__ A, int n, Shared& sh) {
     const int tid = threadIdx.x, nthr = (int)blockDim.x;
     double* vc = sh.v;
@@ -425,6 +425,16 @@ __device__ __noinline__ void tridiagonalise_square(double* __restrict__ A, int n
         if (n >= 2) sh.beta[n - 1] = 0.0;
     }
     __syncthreads();
+}
+
+// The reduction of the factored routes: on the whole matrix where the CTA has a thread for
+// each column of the trailing block, by tiles for larger points (n_v up to MAXN, CTAs of at
+// most NT threads).
+__device__ __noinline__ void tridiagonalise_route(double* __restrict__ A, int n, Shared& sh) {
+    if (n - 1 <= (int)blockDim.x)
+        tridiagonalise_square(A, n, sh);
+    else
+        tridiagonalise(A, n, sh);
 }
 
 // Zt = H^T (rows of Zt are the columns of H = H_0 H_1 ... H_{n-3}), from the
@@ -1133,7 +1143,7 @@ __device__ __noinline__ double solve_lower(const double* __restrict__ L, int m, 
 // the eigenvalues inside.
 __device__ __noinline__ double range_sum(double* __restrict__ C, int m, double xl, double xh, Shared& sh, int* count) {
     const int tid = threadIdx.x;
-    tridiagonalise_square(C, m, sh);
+    tridiagonalise_route(C, m, sh);
     bisect_prepare(m, sh);
     if (tid == 0) {
         sh.misc[0] = max(0, sturm_below(sh.d, sh.p, m, xl) - 1);
@@ -1843,7 +1853,7 @@ solve_kernel(const double* __restrict__ Kfull, const double* __restrict__ KZ, in
         }
         if (!full && !empty) {
             if (routes)
-                tridiagonalise_square(A, n, sh);
+                tridiagonalise_route(A, n, sh);
             else
                 tridiagonalise(A, n, sh);
             bisect_prepare(n, sh);
