@@ -579,8 +579,8 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
     const int nv = P.p.n_v, nvh = P.p.n_vh, n_tot = P.n_tot;
     const int64_t n_tp = n_t / P.B;
     const size_t xs = (size_t)(M + 1) * n_tot * n_tot;
-    int64_t mb = batch_points(P) / (n_tp > 0 ? n_tp : 1);
-    if (mb < 1) mb = 1;
+    const int64_t bt = batch_points(P);
+    const int64_t mb = n_tp < bt ? bt / n_tp : 1;
     // per point: rounding floor scale and range filter [xlo, xhi] of its matrix (fpt), and
     // the matrix's map and norm for the coefficients (pp)
     if ((size_t)(6 * n_t) > h->cap_fpt) {
@@ -698,21 +698,24 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
         CUDA_OR_FAIL(h, dev_alloc(&h->d_zetab, (size_t)mb * (M + 1)));
         h->cap_zetab = (size_t)mb * (M + 1);
     }
-    for (int64_t b0 = 0; b0 < P.B; b0 += mb) {
-        const int64_t b1 = b0 + mb < P.B ? b0 + mb : P.B;
-        const int nbm = (int)(b1 - b0);
-        const int64_t nb = nbm * n_tp;
+    // Chunks of at most bt points (the batch buffers hold no more): all n_tp points of up to
+    // mb matrices, or where a matrix has more than bt, up to bt of one matrix's.
+    for (int64_t g0 = 0, nb; g0 < n_t; g0 += nb) {
+        const int64_t b0 = g0 / n_tp, p0 = g0 - b0 * n_tp;
+        const int64_t np = std::min(n_tp - p0, bt);
+        const int nbm = (int)std::min(mb, P.B - b0);
+        nb = nbm * np;
         // the points of all matrices of the chunk at once: coefficients, assembly, KPM line
         if (share) {
             Scope sc(h, PH_COEFFS);
             CUDA_OR_FAIL(h, launch_expand_coeffs(d_cmu, P.p.damping ? d_cmuh : nullptr, want_ss ? d_cnu : nullptr,
-                                                 d_src, d_sc, n_tp, b0 * n_tp, nb, M, h->d_mu,
+                                                 d_src, d_sc, n_tp, g0, nb, M, h->d_mu,
                                                  P.p.damping ? h->d_muh : nullptr, want_ss ? h->d_nu : nullptr,
                                                  P.stream));
             P.stats.launches++;
         } else {
             Scope sc(h, PH_COEFFS);
-            CUDA_OR_FAIL(h, launch_mu_pp(d_tpts + b0 * n_tp, nb, sigma, d_pp + 3 * b0 * n_tp, M, P.n_theta, P.d_ctab,
+            CUDA_OR_FAIL(h, launch_mu_pp(d_tpts + g0, nb, sigma, d_pp + 3 * g0, M, P.n_theta, P.d_ctab,
                                          h->d_mu, M + 1, P.stream));
             P.stats.launches++;
             if (P.p.damping) {
@@ -752,7 +755,7 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
                     CUDA_OR_FAIL(h, dev_alloc(&h->d_bEmx, (size_t)nbm * ne));
                     h->cap_bEe = (size_t)nbm * ne;
                 }
-                const size_t cb = asm_oz_cslice_bytes(nb, M + 1, ns, n_tp);
+                const size_t cb = asm_oz_cslice_bytes(nb, M + 1, ns, np);
                 if (cb > h->cap_csl) {
                     dev_free(h->d_csl);
                     h->d_csl = nullptr;
@@ -767,34 +770,36 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
                     CUDA_OR_FAIL(h, dev_alloc(&h->d_Et, (size_t)nb));
                     h->cap_Et = (size_t)nb;
                 }
-                CUDA_OR_FAIL(h, launch_asm_oz_xslices(P.d_X + b0 * xs, n_tot, M + 1, h->d_pack, ne, h->d_bEe,
-                                                      h->d_bEmx, h->d_bxsl, ns, P.stream, nbm, xs));
+                if (p0 == 0) {
+                    CUDA_OR_FAIL(h, launch_asm_oz_xslices(P.d_X + b0 * xs, n_tot, M + 1, h->d_pack, ne, h->d_bEe,
+                                                          h->d_bEmx, h->d_bxsl, ns, P.stream, nbm, xs));
+                    P.stats.launches += 3;
+                }
                 CUDA_OR_FAIL(h, launch_asm_oz(muh, M + 1, nb, K + 1, h->d_bxsl, M + 1, h->d_pack, h->d_bEe, ne, n_tot,
-                                              h->d_K, h->d_csl, h->d_Et, P.d_flag, ns, P.stream, n_tp, ne));
+                                              h->d_K, h->d_csl, h->d_Et, P.d_flag, ns, P.stream, np, ne));
                 CUDA_OR_FAIL(h, launch_asm_oz(h->d_nu, M + 1, nb, M + 1, h->d_bxsl, M + 1, h->d_pack, h->d_bEe, nez,
-                                              nv, h->d_KZ, h->d_csl, h->d_Et, P.d_flag, ns, P.stream, n_tp, ne));
-                P.stats.launches += 9;
+                                              nv, h->d_KZ, h->d_csl, h->d_Et, P.d_flag, ns, P.stream, np, ne));
+                P.stats.launches += 6;
             } else {
-                CUDA_OR_FAIL(h, launch_assemble(muh, M + 1, n_tp, K + 1, P.d_X + b0 * xs, n_tot, n_tot, n_tot, h->d_K,
+                CUDA_OR_FAIL(h, launch_assemble(muh, M + 1, np, K + 1, P.d_X + b0 * xs, n_tot, n_tot, n_tot, h->d_K,
                                                 P.stream, nbm, (int64_t)xs));
-                CUDA_OR_FAIL(h, launch_assemble(h->d_nu, M + 1, n_tp, M + 1, P.d_X + b0 * xs, n_tot, nv, nv, h->d_KZ,
+                CUDA_OR_FAIL(h, launch_assemble(h->d_nu, M + 1, np, M + 1, P.d_X + b0 * xs, n_tot, nv, nv, h->d_KZ,
                                                 P.stream, nbm, (int64_t)xs));
                 P.stats.launches += 2;
             }
         }
         {
             Scope sc(h, PH_KPM);
-            CUDA_OR_FAIL(h, launch_kpm_batched(h->d_mu, M + 1, n_tp, nbm, M, P.d_X + b0 * xs, xs, n_tot, h->d_zetab,
-                                               h->d_dos_kpm + b0 * n_tp, P.stream));
+            CUDA_OR_FAIL(h, launch_kpm_batched(h->d_mu, M + 1, np, nbm, M, P.d_X + b0 * xs, xs, n_tot, h->d_zetab,
+                                               h->d_dos_kpm + g0, P.stream));
             P.stats.launches += 2;
         }
         if (want_ss) {
             Scope sc(h, PH_SOLVE);
-            const int64_t nb = (b1 - b0) * n_tp;
             CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, nv, nvh, P.p.tau, 0.0, 0.0,
                                          P.p.damping ? h->d_muh : h->d_mu, M + 1, K, 0.0,
-                                         h->d_solve, h->d_dos_ss + b0 * n_tp, h->d_rank + 2 * b0 * n_tp, P.d_flag,
-                                         P.stream, h->d_fpt + 3 * b0 * n_tp, nullptr,
+                                         h->d_solve, h->d_dos_ss + g0, h->d_rank + 2 * g0, P.d_flag,
+                                         P.stream, h->d_fpt + 3 * g0, nullptr,
                                          (P.p.options & SSM_OPT_PINV) != 0, hybrid_routes(P), h->d_pend));
             P.stats.launches++;
         }
