@@ -366,7 +366,7 @@ stencil_march_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp,
 }
 
 // Float32 stencil step on large 3D grids, by sweeps: a CTA owns an 8 x 8 tile of axes 1
-// and 2 and C 16-byte column chunks, and sweeps a run of planes along axis 0.  A thread
+// and 2 and SWEEP_C 16-byte column chunks, and sweeps a run of planes along axis 0.  A thread
 // keeps its element of planes z - 1, z, z + 1 in registers; the plane's tile and its halo of
 // 32 rows go through shared memory, so an element of V_k is read 1.5 times instead of once
 // per neighbour, and the loads of plane z + 2, of the next halo and of V_{k-1} are in
@@ -378,16 +378,20 @@ stencil_march_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp,
 // beside the Gram products a 64^3 grid of 256 columns takes 0.34 ms a step instead of 0.36.
 // (A ring of asynchronous copies instead of the registers was slower there, 0.35 ms: the
 // Gram CTA holds most of the shared memory; so were sweeps along axis 1 of 2D grids, 68-76
-// ms a call against 61.6 ms on the 256^2 one.)
+// ms a call against 61.6 ms on the 256^2 one.)  Four CTAs an SM, 64 registers a thread: with
+// the 79 that the compiler takes for fewer a call on the 64^3 grid takes 71.3 ms instead of 63.7
+// (256 columns, 128 of them hybrid, degree 300, 400 pencils).
 using Tile3D = SweepTile<8, 8, 1>;
+constexpr uint32_t SWEEP_C = 4;
 
 template <bool PANEL>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(Tile3D::ROWS * SWEEP_C, 4)
 stencil_sweep_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp, float* __restrict__ Vn,
                      const float* __restrict__ diag2, StencilGeom g, float o0, float o1, float o2, float c, float d,
-                     uint32_t nchunk, uint32_t C, uint32_t ngrp, uint32_t nt2, uint32_t planes, PanelOut po) {
+                     uint32_t nchunk, uint32_t ngrp, uint32_t nt2, uint32_t planes, PanelOut po) {
     using ST = Tile3D;
-    extern __shared__ __align__(16) float4 sw[];  // two staged planes
+    constexpr uint32_t C = SWEEP_C, bufsz = ST::PLANE * C;
+    __shared__ float4 sw[2 * bufsz];  // two staged planes
     const int d0 = (int)g.d0, d1 = (int)g.d1, d2 = (int)g.d2;
     const uint32_t grp = blockIdx.x % ngrp, tile = blockIdx.x / ngrp;
     const int b1 = (int)(tile / nt2) * ST::T1, b2 = (int)(tile % nt2) * ST::T2;
@@ -411,7 +415,6 @@ stencil_sweep_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp,
     const bool hok = R.halo && col && q1 >= 0 && q2 >= 0 && (R.ax1 ? on1 : on2);
     const float4* vhal = vc + (hok ? ((size_t)q1 * d2 + q2) * nchunk + cc : 0);
     const uint32_t so = R.own_at() * C + cl, sh = R.halo_at() * C + cl;
-    const uint32_t bufsz = ST::PLANE * C;
     const float4 zero = vzero(0.f);
     auto plane = [&](int z, const float4* v, bool ok) {  // (z may be one past either end of axis 0)
         const int m = axis_at(z, d0, g.per[0] != 0);
@@ -555,32 +558,29 @@ int panel_grid(uint64_t n_rows) {
 }  // namespace
 
 // Launches the sweep kernel where it pays; false where it does not: tiles that do not fit
-// the grid, and blocks below 64 MiB, which the L2 holds (its neighbour reads then cost
-// little, and a run's planes follow one another: 15 to 60 % slower on small grids).
+// the grid, blocks below 64 MiB, which the L2 holds (its neighbour reads then cost
+// little, and a run's planes follow one another: 15 to 60 % slower on small grids), and
+// narrow rows.  A CTA takes four chunks of a row, whole 32-byte sectors whatever the width:
+// one chunk a CTA (all that divides 11, 13, 17, 31 evenly) costs 1.2 to 1.9 times the
+// per-item kernel, three or five up to 1.1 times.  Recurrence and Gram of ten steps on a
+// 128^3 grid, by tiles of four chunks and by items: 16.3 and 16.6 ms at 33 chunks, 25.2 and
+// 26.8 at 51, 30.3 and 33.9 at 64; 14.4 and 14.4 at 29, 9.5 and 9.2 at 19, 5.1 and 4.8 at 9;
+// without idle columns 9.3 and 9.4 at 20, 5.6 and 5.7 at 12, 4.6 and 4.5 at 8.
 static bool sweep_step(const StencilGeom& g, int64_t n, uint32_t nchunk, const float* Vc, const float* Vp, float* Vn,
                        const float* diag2, float o0, float o1, float o2, float c, float d, PanelOut po,
                        cudaStream_t s) {
     using ST = Tile3D;
-    if ((uint64_t)n * nchunk * 16 < (64ull << 20)) return false;
-    // chunks a CTA: the fewest idle columns, four on ties
-    uint32_t C = 4, best = ~0u;
-    for (const uint32_t q : {4u, 5u, 6u, 3u, 7u, 8u, 2u, 1u}) {
-        const uint32_t idle = (nchunk + q - 1) / q * q - nchunk;
-        if (idle < best) {
-            best = idle;
-            C = q;
-        }
-    }
+    constexpr uint32_t C = SWEEP_C;
+    if ((uint64_t)n * nchunk * 16 < (64ull << 20) || nchunk < (nchunk % C ? 24u : 12u)) return false;
     const uint32_t ngrp = (nchunk + C - 1) / C;
     // about sixteen 256-thread CTAs an SM over the launch (its last wave is then a small
     // part), at least eight planes a run
     const SweepRuns w = sweep_runs<ST>(g.d0, g.d1, g.d2, ngrp, (uint64_t)device_sms() * 16 * 256 / (ST::ROWS * C), 8);
     if (!w.nseg) return false;
     const dim3 grid(ngrp * w.nt1 * w.nt2, w.nseg);
-    const size_t smem = (size_t)2 * ST::PLANE * C * 16;
     const auto kernel = po.base ? stencil_sweep_kernel<true> : stencil_sweep_kernel<false>;
-    kernel<<<grid, ST::ROWS * C, smem, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, g, o0, o1, o2, c, d, nchunk, C, ngrp, w.nt2,
-                                            w.planes, po);
+    kernel<<<grid, ST::ROWS * C, 0, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, g, o0, o1, o2, c, d, nchunk, ngrp, w.nt2,
+                                         w.planes, po);
     return true;
 }
 
