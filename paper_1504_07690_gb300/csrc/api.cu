@@ -830,7 +830,7 @@ cudaError_t record_batched_moments(Plan& P, cudaStream_t cs, cudaStream_t cs2) {
             cudaError_t r = launch_gram_tc(P.d_panel[j % 3], Vc ? P.d_panel[(j + 2) % 3] : nullptr, P.n_tot, P.n,
                                            P.tc_ne, P.tc_no, P.d_part_tc, P.d_flag, cs2, P.d_slabs, gram_both(P));
             if (r != cudaSuccess) return r;
-            return launch_reduce_tc_seg(P.d_part_tc, P.tc_ne, P.n_tot, B, P.d_slabseg, P.d_ring_sum,
+            return launch_reduce_tc_seg(P.d_part_tc, P.tc_ne, P.n_tot, B, P.d_slabseg, P.n_many, P.d_ring_sum,
                                         P.d_ring_sum + (size_t)B * nn, P.d_X, xs, step, cs2);
         }
         for (int b = 0; b < B; ++b) {
@@ -875,9 +875,11 @@ cudaError_t record_batched_moments(Plan& P, cudaStream_t cs, cudaStream_t cs2) {
 }
 
 // Gram slab table of a batched plan: each matrix's panels in ~equal slabs of at most
-// `pe` (Ge) and `po` (Go) panels, Ge slabs first; seg: per-matrix slab ranges.
+// `pe` (Ge) and `po` (Go) panels, Ge slabs first; seg: per-matrix slab ranges, then the
+// matrices in the order of their reduction, the n_many of more than MANY_SLABS Ge slabs first.
+constexpr int MANY_SLABS = 4;
 void build_slabs(const int64_t* row_off, int B, int64_t pe, int64_t po, std::vector<int2>& slabs,
-                 std::vector<int>& seg, int& ne) {
+                 std::vector<int>& seg, int& ne, int& n_many) {
     slabs.clear();
     seg.assign(2 * (B + 1), 0);
     for (int pass = 0; pass < 2; ++pass) {
@@ -895,6 +897,13 @@ void build_slabs(const int64_t* row_off, int B, int64_t pe, int64_t po, std::vec
         seg[pass * (B + 1) + B] = (int)slabs.size() - base;
         if (pass == 0) ne = (int)slabs.size();
     }
+    n_many = 0;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int b = 0; b < B; ++b)
+            if ((seg[b + 1] - seg[b] > MANY_SLABS) == (pass == 0)) {
+                seg.push_back(b);
+                if (pass == 0) ++n_many;
+            }
 }
 
 // Install the slab table with slabs of `div`-th of the default size (the default: one Ge
@@ -911,7 +920,7 @@ cudaError_t install_slabs(Plan& P, int div) {
     std::vector<int2> slabs;
     std::vector<int> seg;
     int ne = 0;
-    build_slabs(P.h_row_off, P.B, pe, po, slabs, seg, ne);
+    build_slabs(P.h_row_off, P.B, pe, po, slabs, seg, ne, P.n_many);
     const int no = (int)slabs.size() - ne;
     const size_t need = gram_tc_partial_floats(ne, no, P.n_tot);
     if (slabs.size() > P.cap_slabs || need > P.cap_part_tc) {
@@ -973,7 +982,7 @@ cudaError_t autotune_gram(Plan& P) {
                 err = launch_gram_tc(P.d_panel[1], P.d_panel[0], P.n_tot, P.n, P.tc_ne, P.tc_no, P.d_part_tc,
                                      P.d_flag, s2, P.d_slabs, gram_both(P));
             if (err == cudaSuccess)
-                err = launch_reduce_tc_seg(P.d_part_tc, P.tc_ne, P.n_tot, P.B, P.d_slabseg, P.d_ring_sum,
+                err = launch_reduce_tc_seg(P.d_part_tc, P.tc_ne, P.n_tot, P.B, P.d_slabseg, P.n_many, P.d_ring_sum,
                                            P.d_ring_sum + (size_t)P.B * nn, P.d_X, xs, 0, s2);
             if (err == cudaSuccess)
                 err = launch_csr_step_f32(P, (const float*)P.d_V[0], (const float*)P.d_V[1], (float*)P.d_V[2], 1.f,

@@ -38,6 +38,8 @@
 // for its MMAs, frees TMEM and returns.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "internal.h"
 #include "tcgen05.cuh"
 
@@ -412,14 +414,14 @@ __global__ void moments_tc_batch_kernel(const double* __restrict__ ge, const dou
     }
 }
 
-// Batched plans: matrix b = blockIdx.y sums its own slabs (Ge slabs [se[b],
-// se[b+1]), Go slabs [so[b], so[b+1])), in the fixed order of sum_tc_kernel.
+// Batched plans: the blockIdx.y-th matrix b of `order` (NULL: b itself) sums its own slabs
+// (Ge slabs [se[b], se[b+1]), Go slabs [so[b], so[b+1])), in the fixed order of sum_tc_kernel.
 __global__ void __launch_bounds__(256)
-sum_tc_seg_kernel(const float* __restrict__ pe, const float* __restrict__ po, const int* __restrict__ seg, int B,
-                  int n_tot, bool odd, double* __restrict__ ge, double* __restrict__ go) {
+sum_tc_seg_kernel(const float* __restrict__ pe, const float* __restrict__ po, const int* __restrict__ seg,
+                  const int* __restrict__ order, int B, int n_tot, bool odd, double* __restrict__ ge, double* __restrict__ go) {
     __shared__ double se_[8][32], so_[8][32];
     const size_t nn = (size_t)n_tot * n_tot;
-    const int b = blockIdx.y;
+    const int b = order ? order[blockIdx.y] : (int)blockIdx.y;
     const int e0s = seg[b], e1s = seg[b + 1], o0s = seg[B + 1 + b], o1s = seg[B + 2 + b];
     double* gq = ge + (size_t)b * nn;
     double* oq = go + (size_t)b * nn;
@@ -448,10 +450,11 @@ sum_tc_seg_kernel(const float* __restrict__ pe, const float* __restrict__ po, co
     }
 }
 
-__global__ void moments_tc_seg_kernel(const double* __restrict__ ge, const double* __restrict__ go, int n_tot,
-                                      double* __restrict__ X, size_t xstride, int step) {
+__global__ void moments_tc_seg_kernel(const double* __restrict__ ge, const double* __restrict__ go,
+                                      const int* __restrict__ order, int n_tot, double* __restrict__ X, size_t xstride,
+                                      int step) {
     const size_t nn = (size_t)n_tot * n_tot;
-    const int b = blockIdx.y;
+    const int b = order ? order[blockIdx.y] : (int)blockIdx.y;
     const double* gq = ge + (size_t)b * nn;
     const double* oq = go + (size_t)b * nn;
     double* Xb = X + (size_t)b * xstride;
@@ -471,9 +474,9 @@ __global__ void moments_tc_seg_kernel(const double* __restrict__ ge, const doubl
     }
 }
 
-// The same sums and the moments of a step in one launch, for batches of small matrices: one
-// thread an element pair (i, j), (j, i), the chains of sum_tc_kernel one after the other (an
-// empty chain adds nothing).
+// The same sums and the moments of a step in one launch, for small matrices (the order's
+// from n_many on): one thread an element pair (i, j), (j, i), the chains of sum_tc_kernel one
+// after the other (an empty chain adds nothing).
 __device__ __forceinline__ double chain_sum(const float* __restrict__ p, size_t nn, size_t e, int k0, int k1) {
     double s = 0.0;
     const int k8 = min(k1, k0 + 8);
@@ -487,10 +490,10 @@ __device__ __forceinline__ double chain_sum(const float* __restrict__ p, size_t 
 }
 
 __global__ void __launch_bounds__(256)
-step_tc_seg_kernel(const float* __restrict__ pe, const float* __restrict__ po, const int* __restrict__ seg, int B,
-                   int n_tot, double* __restrict__ X, size_t xstride, int step) {
+step_tc_seg_kernel(const float* __restrict__ pe, const float* __restrict__ po, const int* __restrict__ seg,
+                   const int* __restrict__ order, int B, int n_tot, double* __restrict__ X, size_t xstride, int step) {
     const size_t nn = (size_t)n_tot * n_tot;
-    const int b = blockIdx.y;
+    const int b = order ? order[blockIdx.y] : (int)blockIdx.y;
     const int e0 = seg[b], e1 = seg[b + 1], o0 = seg[B + 1 + b], o1 = seg[B + 2 + b];
     double* Xb = X + (size_t)b * xstride;
     const unsigned npair = (unsigned)n_tot * (n_tot + 1) / 2;
@@ -673,30 +676,36 @@ cudaError_t launch_reduce_tc_batch(const float* ring, int n_e, int n_o, int n_to
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_tc_seg(const float* part, int n_e, int n_tot, int B, const int* seg, double* ge,
+// Matrices of few slabs: a thread an element.  The eight warps an element of the other
+// kernels spend the float64 pipe on converting and adding zeros there (1100 matrices of one
+// slab, n_tot = 32: 125 us and 14 us for the moments, against 24 us); with more slabs they
+// share the loads.  Each matrix goes by its own slabs: one of 200000 rows (550 slabs) beside
+// 300 of 100, 30 steps: n_tot = 8 3.25 ms with a thread an element for all, 1.68 with eight
+// warps for all, 1.77 so; 32: 7.0, 4.7 and 4.0; 64: 10.4, 11.0 and 7.4; 200: 39.8, 63.0 and
+// 31.1.  1000 of 300 beside three of 100000: 32 7.4, 10.5 and 7.3.
+cudaError_t launch_reduce_tc_seg(const float* part, int n_e, int n_tot, int B, const int* seg, int n_many, double* ge,
                                  double* go, double* X, size_t xstride, int step, cudaStream_t s) {
     const int64_t nn = (int64_t)n_tot * n_tot;
-    // Few slabs a matrix and many matrices: a thread an element.  The eight warps an element of
-    // the other path spend the float64 pipe on converting and adding zeros there (1100 matrices
-    // of one slab, n_tot = 32: 125 us and 14 us for the moments, against 24 us); with more
-    // slabs than warps they share the loads.
-    if (n_e <= (int64_t)4 * B) {
+    const float* po = part + (size_t)n_e * nn;
+    const int* order = n_many > 0 && n_many < B ? seg + 2 * (B + 1) : nullptr;  // (one kind only: any order)
+    if (n_many < B) {
         int64_t pb = (nn / 2 + n_tot + 255) / 256;
         if (pb > 64) pb = 64;
-        step_tc_seg_kernel<<<dim3((unsigned)pb, (unsigned)B), 256, 0, s>>>(part, part + (size_t)n_e * nn, seg, B, n_tot,
-                                                                         X, xstride, step);
-        return cudaGetLastError();
+        step_tc_seg_kernel<<<dim3((unsigned)pb, (unsigned)(B - n_many)), 256, 0, s>>>(
+            part, po, seg, order ? order + n_many : nullptr, B, n_tot, X, xstride, step);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
-    int64_t sb = (nn + 31) / 32;
-    if (sb > 64) sb = 64;
-    dim3 sg((unsigned)sb, (unsigned)B);
-    sum_tc_seg_kernel<<<sg, 256, 0, s>>>(part, part + (size_t)n_e * nn, seg, B, n_tot, step >= 0, ge, go);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    int64_t mb = (nn + 255) / 256;
-    if (mb > 64) mb = 64;
-    dim3 mg((unsigned)mb, (unsigned)B);
-    moments_tc_seg_kernel<<<mg, 256, 0, s>>>(ge, go, n_tot, X, xstride, step);
+    if (n_many > 0) {
+        // at most 64 CTAs a matrix, more where few matrices would leave SMs idle
+        const int64_t cap = std::max<int64_t>(64, (int64_t)device_sms() * 8 / n_many);
+        const int64_t sb = std::min((nn + 31) / 32, cap), mb = std::min((nn + 255) / 256, cap);
+        sum_tc_seg_kernel<<<dim3((unsigned)sb, (unsigned)n_many), 256, 0, s>>>(part, po, seg, order, B, n_tot, step >= 0,
+                                                                             ge, go);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        moments_tc_seg_kernel<<<dim3((unsigned)mb, (unsigned)n_many), 256, 0, s>>>(ge, go, order, n_tot, X, xstride, step);
+    }
     return cudaGetLastError();
 }
 

@@ -133,7 +133,8 @@ struct Plan {
     double* d_beta_row64 = nullptr;    // per-row beta of the folded map (batched CSR)
     float* d_beta_row32 = nullptr;
     int2* d_slabs = nullptr;           // tensor-core Gram slab table [n_e + n_o] (panel ranges)
-    int* d_slabseg = nullptr;          // per-matrix slab ranges: se[B+1], so[B+1]
+    int* d_slabseg = nullptr;          // per-matrix slab ranges: se[B+1], so[B+1]; order[B]
+    int n_many = 0;                    // matrices of many slabs (the first of the order)
     double* d_x0max = nullptr;         // per-matrix max_i X_0[i][i] (B)
     int64_t* d_boff = nullptr;         // row_off (B + 1), then the matrices' offsets in W (B + 1)
     cudaStream_t cap_stream = nullptr; // capture streams of the batched recurrence graph (the
@@ -253,9 +254,9 @@ int gram_tc_groups(int n_tot);  // 8-column groups of a panel
 cudaError_t launch_gram_tc(const uint8_t* PX, const uint8_t* PY, int n_tot, int64_t n_rows, int n_e, int n_o,
                            float* part, int* flag, cudaStream_t s, const int2* slabs = nullptr, bool both = false);
 // Batched plans: per-matrix slab sums (matrix b owns Ge slabs [se[b], se[b+1]) and Go
-// slabs [so[b], so[b+1]); seg = se (B+1) followed by so (B+1)) and the moments of step
-// `step` (-1: X_0) into X + b * xstride.
-cudaError_t launch_reduce_tc_seg(const float* part, int n_e, int n_tot, int B, const int* seg, double* ge,
+// slabs [so[b], so[b+1]); seg = se (B+1), so (B+1), then the matrices' order, the n_many of
+// many slabs first) and the moments of step `step` (-1: X_0) into X + b * xstride.
+cudaError_t launch_reduce_tc_seg(const float* part, int n_e, int n_tot, int B, const int* seg, int n_many, double* ge,
                                  double* go, double* X, size_t xstride, int step, cudaStream_t s);
 cudaError_t launch_reduce_tc(const float* part, int n_e, int n_o, int n_tot, double* X, int step, cudaStream_t s);
 // Moments of steps k0..k0+nk-1 from a ring of nk partial slots (float64 scratch ge, go: nk x n_tot^2 each).
