@@ -221,8 +221,11 @@ ssm_status ssm_moments(ssm_plan_t plan, const double* W, int64_t ldw, double* mo
  * dos_ss: RESS-DGC estimate of Tr g_sigma^{M/2}(tI - A) (Theorem 4);
  * dos_kpm: DGC/KPM estimate sum_{l<=M} mu_l(t) Tr X_l / n_tot.  Either output
  * may be NULL.  rank (nullable): n_t x 2 int32, the kept ranks after Alg. 4's
- * truncation and after its range filter.  Returns SSM_ESTATE without
- * moments, SSM_EINVAL for sigma <= 0 or n_t < 0 (n_t = 0 is a no-op). */
+ * truncation and after its range filter.  The same call on the same moments
+ * repeats bit for bit; a point's estimate may differ in the last bits between
+ * calls of few and of many points (the order of the sums in its solve goes by
+ * n_t).  Returns SSM_ESTATE without moments, SSM_EINVAL for sigma <= 0 or
+ * n_t < 0 (n_t = 0 is a no-op). */
 ssm_status ssm_dos(ssm_plan_t plan, const double* t, int64_t n_t, double sigma,
                    double* dos_ss, double* dos_kpm, int32_t* rank);
 
@@ -237,13 +240,13 @@ ssm_status ssm_dos(ssm_plan_t plan, const double* t, int64_t n_t, double sigma,
  * step is added into all blocks Z_i: N n_v n_t (M+1) float64 multiply-adds and
  * n_t Gram pairs, for few sweep points.  The blocks of as many points as fit in
  * half of the free device memory are held at a time; further chunks of points
- * rerun the recurrence.  W: N x n_v float64 (host or device, leading
- * dimension ldw >= n_v).  t: n_t points (host or device).  dos (n_t) and rank
- * (n_t x 2 int32, ranks after the truncation and after the range filter) may
- * each be NULL, on host or device.  Needs a single-operator SSM_FP64 plan
- * with n_vh = 0 (SSM_EINVAL otherwise); independent of ssm_moments (the
- * plan's moments are left as they are).  SSM_ENONFINITE if W is not finite,
- * SSM_ENOMEM if one block Z does not fit. */
+ * rerun the recurrence (the results do not depend on the chunks).  W: N x n_v
+ * float64 (host or device, leading dimension ldw >= n_v).  t: n_t points (host
+ * or device).  dos (n_t) and rank (n_t x 2 int32, ranks after the truncation
+ * and after the range filter) may each be NULL, on host or device.  Needs a
+ * single-operator SSM_FP64 plan with n_vh = 0 (SSM_EINVAL otherwise);
+ * independent of ssm_moments (the plan's moments are left as they are).
+ * SSM_ENONFINITE if W is not finite, SSM_ENOMEM if one block Z does not fit. */
 ssm_status ssm_dos_explicit(ssm_plan_t plan, const double* W, int64_t ldw, const double* t, int64_t n_t,
                             double sigma, double* dos, int32_t* rank);
 

@@ -553,7 +553,7 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
                     perm = h->d_perm;
                 }
             }
-            CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, nv, nvh, P.p.tau, xlo, xhi, muh, M + 1, K,
+            CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, n_t, nv, nvh, P.p.tau, xlo, xhi, muh, M + 1, K,
                                          floor_scale, h->d_solve, h->d_dos_ss + t0, h->d_rank + 2 * t0,
                                          P.d_flag, P.stream, nullptr, perm, (P.p.options & SSM_OPT_PINV) != 0,
                                          hybrid_routes(P), h->d_pend));
@@ -796,7 +796,7 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
         }
         if (want_ss) {
             Scope sc(h, PH_SOLVE);
-            CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, nv, nvh, P.p.tau, 0.0, 0.0,
+            CUDA_OR_FAIL(h, launch_solve(h->d_K, h->d_KZ, nb, n_t, nv, nvh, P.p.tau, 0.0, 0.0,
                                          P.p.damping ? h->d_muh : h->d_mu, M + 1, K, 0.0,
                                          h->d_solve, h->d_dos_ss + g0, h->d_rank + 2 * g0, P.d_flag,
                                          P.stream, h->d_fpt + 3 * g0, nullptr,
@@ -2077,7 +2077,7 @@ ssm_status ssm_dos_explicit(ssm_plan_t h, const double* W, int64_t ldw, const do
         }
         {
             Scope sc(h, PH_SOLVE);
-            CUDA_OR_FAIL(h, launch_solve(d_K, d_KZ, nc, nv, 0, P.p.tau, xlo, xhi, mu_c, M + 1, M, floor_scale,
+            CUDA_OR_FAIL(h, launch_solve(d_K, d_KZ, nc, n_t, nv, 0, P.p.tau, xlo, xhi, mu_c, M + 1, M, floor_scale,
                                          h->d_solve, d_dos + t0, d_rank + 2 * t0, P.d_flag, st, nullptr, nullptr,
                                          (P.p.options & SSM_OPT_PINV) != 0));
             P.stats.launches++;

@@ -357,10 +357,13 @@ cudaError_t launch_asm_oz(const double* coef, int ldc, int64_t n_t, int L, const
 // pend (nullable, n_t + 1 ints): room for the points that the warp-per-point kernel of
 // small n_v leaves to the CTA-per-point one.
 // hyb: hybrid columns take the factored routes (mixed plans with n_vh > 0).
+// n_call: points of the whole call, of which these are the n_t of one chunk; the shape of the
+// launch, and with it the order of a point's sums, goes by n_call, so that a point's result
+// does not depend on how memory cuts the call into chunks.
 size_t solve_workspace_bytes(int n_v, bool hyb);
 // floor(t) = floor_scale * sum_{l<=K} (l+1) |mu[t][l]| (see ssm_params.eps_floor).  floor_pt
 // (nullable): per point (floor_scale, xlo, xhi), replacing the scalars (batched plans).
-cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int n_v, int n_vh,
+cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int64_t n_call, int n_v, int n_vh,
                          double tau, double xlo, double xhi, const double* mu, int ldmu, int K,
                          double floor_scale, void* work, double* dos, int32_t* rank, int* flag,
                          cudaStream_t s, const double* floor_pt = nullptr, const int32_t* perm = nullptr,
@@ -369,7 +372,7 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
 // slots of one wave, the length of a schedule.
 int64_t solve_slots(int n_v, bool hyb, int64_t n_t);
 // Whether a launch_solve with room in `pend` runs the warp-per-point kernel first.
-bool solve_uses_small(int64_t n_t, int n_v, int n_vh, bool pinv);
+bool solve_uses_small(int64_t n_call, int n_v, int n_vh, bool pinv);
 // Schedule (perm, solve_slots(n_v) entries) of the next solve launch over n_t points
 // from the kept ranks of the previous launch over the same number of points; a
 // heuristic for speed only: every point is solved whatever perm holds.

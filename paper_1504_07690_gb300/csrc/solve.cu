@@ -12,15 +12,15 @@ namespace {
 // per SM).
 int solve_threads(int n_v) { return n_v <= 128 ? 128 : NT; }
 
-// ... but a launch of few points lasts as long as its slowest ones, and a float64 fma holds
+// ... but a call of few points lasts as long as its slowest ones, and a float64 fma holds
 // its warp for 65 cycles of which the pipe is busy 16: eight warps a point, for points with
 // hybrid columns up to four an SM (400 points of n_v = 128, n_vh = 128: 12.4 ms against 18.3;
 // 600 of n_v = 100: 7.5 against 8.6, 900: no gain), without up to two (20 points of n_v = 100:
 // 5.1 against 6.4; where every point keeps a part of its directions 300 take 7.4 against 7.8,
 // 450 9.3 against 9.1).  The step-by-step route of float64 plans keeps its sums' order.
-int solve_threads(int n_v, int n_vh, bool hyb, int64_t n_t) {
+int solve_threads(int n_v, int n_vh, bool hyb, int64_t n_call) {
     const int per_sm = hyb ? (n_v > 32 ? 4 : 0) : (n_vh == 0 && n_v > 64 ? 2 : 0);
-    return n_t <= (int64_t)per_sm * device_sms() ? NT : solve_threads(n_v);
+    return n_call <= (int64_t)per_sm * device_sms() ? NT : solve_threads(n_v);
 }
 
 // CTAs with a private workspace: 4 x (256 / threads) per SM to overlap the
@@ -99,9 +99,9 @@ __global__ void solve_schedule_kernel(const int32_t* __restrict__ rank_prev, int
     for (int64_t b = threadIdx.x; b < slots; b += blockDim.x) perm_out[b] = perm[b] == -2 ? -1 : perm[b];
 }
 
-cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int n_v, int n_vh, double tau,
-                         double xlo, double xhi, const double* mu, int ldmu, int K, double floor_scale, void* work,
-                         double* dos, int32_t* rank, int* flag, cudaStream_t s, const double* floor_pt,
+cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int64_t n_call, int n_v, int n_vh,
+                         double tau, double xlo, double xhi, const double* mu, int ldmu, int K, double floor_scale,
+                         void* work, double* dos, int32_t* rank, int* flag, cudaStream_t s, const double* floor_pt,
                          const int32_t* perm, bool pinv, bool hyb, int32_t* pend) {
     if (n_t <= 0) return cudaSuccess;
     if (n_v > MAXN) return cudaErrorInvalidValue;
@@ -111,22 +111,23 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
     if (e != cudaSuccess) return e;
     int64_t grid = workspace_ctas(n_v, hyb), n_slot = n_t;
     if (perm) {
-        n_slot = solve_slots(n_v, hyb, n_t);
+        n_slot = solve_slots(n_v, hyb, n_call);
         if (n_slot < n_t || n_slot > grid) return cudaErrorInvalidValue;
     }
     if (grid > n_slot) grid = n_slot;
     // small points without hybrid columns: a warp each; what is left goes on
     const int32_t* n_dev = nullptr;
-    if (pend && solve_uses_small(n_t, n_v, n_vh, pinv)) {
+    if (pend && solve_uses_small(n_call, n_v, n_vh, pinv)) {
         e = launch_solve_small(Kfull, KZ, n_t, n_v, tau, xlo, xhi, mu, ldmu, K, floor_scale, dos, rank, floor_pt, pend,
                                s);
         if (e != cudaSuccess) return e;
         n_dev = pend;
         perm = pend + 1;
     }
-    kernel<<<(int)grid, solve_threads(n_v, n_vh, hyb, n_t), smem, s>>>(Kfull, KZ, n_t, n_v, n_vh, tau, xlo, xhi, mu,
-                                                                       ldmu, K, floor_scale, (double*)work, dos, rank,
-                                                                       flag, floor_pt, perm, n_slot, pinv, n_dev);
+    kernel<<<(int)grid, solve_threads(n_v, n_vh, hyb, n_call), smem, s>>>(Kfull, KZ, n_t, n_v, n_vh, tau, xlo, xhi, mu,
+                                                                          ldmu, K, floor_scale, (double*)work, dos,
+                                                                          rank, flag, floor_pt, perm, n_slot, pinv,
+                                                                          n_dev);
     return cudaGetLastError();
 }
 
@@ -134,8 +135,8 @@ cudaError_t launch_solve(const double* Kfull, const double* KZ, int64_t n_t, int
 // either way, and a warp's serial chain is the longer one (n_v = 32: 1.06 against 1.31 ms
 // at 73 points, 1.19 against 1.34 at 600, 1.79 against 1.44 at 1200; n_v = 16: 0.42
 // against 0.55, 0.60 against 0.59, 0.72 against 0.65).
-bool solve_uses_small(int64_t n_t, int n_v, int n_vh, bool pinv) {
-    return n_v <= SOLVE_SMALL_N && n_vh == 0 && !pinv && n_t >= (int64_t)8 * device_sms();
+bool solve_uses_small(int64_t n_call, int n_v, int n_vh, bool pinv) {
+    return n_v <= SOLVE_SMALL_N && n_vh == 0 && !pinv && n_call >= (int64_t)8 * device_sms();
 }
 
 int64_t solve_slots(int n_v, bool hyb, int64_t n_t) {
