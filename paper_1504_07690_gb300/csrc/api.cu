@@ -537,8 +537,8 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
             const bool single = t0 == 0 && nb == n_t;
             const int32_t* perm = nullptr;
             // (no use where every point runs the serial QL chains, or a warp-size kernel first)
-            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P)) &&
-                !solve_uses_small(n_t, nv, nvh, (P.p.options & SSM_OPT_PINV) != 0)) {
+            const bool small = solve_uses_small(n_t, nv, nvh, (P.p.options & SSM_OPT_PINV) != 0);
+            if (single && h->sched_nt == n_t && (nvh == 0 || hybrid_routes(P)) && !small) {
                 const int64_t slots = solve_slots(nv, hybrid_routes(P), n_t);
                 if (slots >= n_t) {
                     if ((size_t)slots > h->cap_perm) {
@@ -557,7 +557,7 @@ ssm_status dos_dev(ssm_plan_s* h, const double* d_tpts, int64_t n_t, double sigm
                                          floor_scale, h->d_solve, h->d_dos_ss + t0, h->d_rank + 2 * t0,
                                          P.d_flag, P.stream, nullptr, perm, (P.p.options & SSM_OPT_PINV) != 0,
                                          hybrid_routes(P), h->d_pend));
-            P.stats.launches++;
+            P.stats.launches += small ? 2 : 1;
             h->sched_nt = single ? n_t : 0;
         }
         {
@@ -801,7 +801,7 @@ ssm_status dos_dev_batched(ssm_plan_s* h, const double* d_tpts, int64_t n_t, dou
                                          h->d_solve, h->d_dos_ss + g0, h->d_rank + 2 * g0, P.d_flag,
                                          P.stream, h->d_fpt + 3 * g0, nullptr,
                                          (P.p.options & SSM_OPT_PINV) != 0, hybrid_routes(P), h->d_pend));
-            P.stats.launches++;
+            P.stats.launches += solve_uses_small(n_t, nv, nvh, (P.p.options & SSM_OPT_PINV) != 0) ? 2 : 1;
         }
     }
     return SSM_OK;
