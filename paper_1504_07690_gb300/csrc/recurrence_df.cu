@@ -106,7 +106,7 @@ __device__ __forceinline__ unsigned long long bound_bits(float h) {
     return (unsigned long long)__double_as_longlong((double)fabsf(h) * (1.0 + 0x1.0p-22));
 }
 
-// A CTA of (nch, ty) threads takes DF_ROWS ty consecutive rows: thread (x, y) owns the
+// A CTA of (nch, ty) threads takes up to DF_ROWS ty consecutive rows: thread (x, y) owns the
 // 16-byte column chunk x (four columns, float4 loads and stores of each plane) of rows y,
 // y + ty, ..., so no thread idles whatever the number of columns; it keeps the column
 // maxima of its rows in registers, and the CTA combines them in shared memory before one
@@ -234,12 +234,12 @@ stencil_step_df_kernel(DfBlock Vc, DfBlock Vp, const float* __restrict__ dgh, co
 __global__ void __launch_bounds__(DF_THREADS)
 csr_step_df_kernel(DfBlock Vc, DfBlock Vp, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
                    const float* __restrict__ vh, const float* __restrict__ vl, F2 beta, float c, float d,
-                   uint32_t ld, uint32_t n_cols, uint32_t n_rows, DfOut out) {
+                   uint32_t ld, uint32_t n_cols, uint32_t n_rows, uint32_t per, DfOut out) {
     const uint32_t cx = threadIdx.x, nch = blockDim.x;
     const pair32 c2 = pair_of(c, c);
     float mv[4] = {0.f, 0.f, 0.f, 0.f}, mu[4] = {0.f, 0.f, 0.f, 0.f};
-    const uint32_t first = blockIdx.x * (DF_ROWS * blockDim.y) + threadIdx.y;
-    for (uint32_t k = 0; k < DF_ROWS; ++k) {
+    const uint32_t first = blockIdx.x * (per * blockDim.y) + threadIdx.y;
+    for (uint32_t k = 0; k < per; ++k) {
         const uint32_t i = first + k * blockDim.y;
         if (i >= n_rows) break;
         const size_t i4 = (size_t)i * nch + cx;
@@ -314,16 +314,25 @@ cudaError_t launch_step_df(const Plan& P, const void* Vc, const void* Vp, void* 
     if (P.ld > 4 * DF_MAXCH || (P.ld & 3)) return cudaErrorInvalidValue;  // a thread per 4 columns
     const uint32_t nch = (uint32_t)P.ld / 4;
     const dim3 nt(nch, DF_THREADS / nch);
-    const uint32_t rows = DF_ROWS * nt.y;
-    const unsigned grid = (unsigned)((P.n + rows - 1) / rows);
+    auto ctas = [&](uint32_t per) { return (unsigned)((P.n + per * nt.y - 1) / (per * nt.y)); };
     if (P.is_stencil) {
+        const unsigned grid = ctas(DF_ROWS);
         stencil_step_df_kernel<<<grid, nt, 0, s>>>(
             vc, vp, P.d_diag32, P.d_diag32lo, P.geom, split_f2(P.off64[0]), split_f2(P.off64[1]),
             split_f2(P.off64[2]), c, d, (uint32_t)P.ld, (uint32_t)P.n_tot, (uint32_t)P.n, o);
     } else {
-        csr_step_df_kernel<<<grid, nt, 0, s>>>(vc, vp, P.d_rowptr, P.d_colind, P.d_val32, P.d_val32lo,
-                                                          split_f2(P.beta), c, d, (uint32_t)P.ld,
-                                                          (uint32_t)P.n_tot, (uint32_t)P.n, o);
+        // A CSR row is a serial chain of gathers, so a thread takes as many rows, up to
+        // DF_ROWS, as leave two CTAs an SM.  Narrow blocks of eight rows a thread put few
+        // CTAs on the chip: 30 steps of 30000 rows of 8 columns (30 CTAs) 5.2 ms, 1.7 with a
+        // row a thread; 40 columns 4.1 and 2.1 with two rows; 300000 rows of one column 17.6
+        // and 8.7.  Where eight rows leave enough, fewer cost the Gram products beside them
+        // more than they gain (30011 rows of 160 columns, degree 200: 19.6 ms a call, 20.6 with
+        // two rows; 300000 of 100: 32.6, 35.1 with one).
+        uint32_t per = DF_ROWS;
+        while (per > 1 && ctas(per) < 2u * (unsigned)device_sms()) per /= 2;
+        csr_step_df_kernel<<<ctas(per), nt, 0, s>>>(vc, vp, P.d_rowptr, P.d_colind, P.d_val32, P.d_val32lo,
+                                                    split_f2(P.beta), c, d, (uint32_t)P.ld, (uint32_t)P.n_tot,
+                                                    (uint32_t)P.n, per, o);
     }
     return cudaGetLastError();
 }
