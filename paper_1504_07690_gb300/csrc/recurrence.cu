@@ -559,19 +559,31 @@ int panel_grid(uint64_t n_rows) {
 
 // Launches the sweep kernel where it pays; false where it does not: tiles that do not fit
 // the grid, blocks below 64 MiB, which the L2 holds (its neighbour reads then cost
-// little, and a run's planes follow one another: 15 to 60 % slower on small grids), and
-// narrow rows.  A CTA takes four chunks of a row, whole 32-byte sectors whatever the width:
+// little, and a run's planes follow one another: 15 to 60 % slower on small grids), narrow
+// rows, and small planes with ragged tiles.
+//
+// A CTA takes four chunks of a row, whole 32-byte sectors whatever the width:
 // one chunk a CTA (all that divides 11, 13, 17, 31 evenly) costs 1.2 to 1.9 times the
 // per-item kernel, three or five up to 1.1 times.  Recurrence and Gram of ten steps on a
 // 128^3 grid, by tiles of four chunks and by items: 16.3 and 16.6 ms at 33 chunks, 25.2 and
 // 26.8 at 51, 30.3 and 33.9 at 64; 14.4 and 14.4 at 29, 9.5 and 9.2 at 19, 5.1 and 4.8 at 9;
 // without idle columns 9.3 and 9.4 at 20, 5.6 and 5.7 at 12, 4.6 and 4.5 at 8.
+//
+// Planes of 8 MiB outlast the caches between the uses of a row, and the sweep gains with
+// tiles a quarter past the edges (60 x 250 x 250 of 128 columns: 26.1 and 29.9 ms; 128 x 121
+// x 121 of 256: 28.1 and 29.2).  Smaller ones are read no more often by items, and where the
+// step also writes panels every idle row shows (500 x 60 x 60 of 128: 12.9 and 12.4; 500 x 57 x
+// 57: 12.0 and 11.2), so there the tiles have to fit to 1/32 (128^3 of 64 columns: 7.35 and
+// 7.45; 64^3 of 256: 3.95 and 4.03).  Without panels a step of 100^3 of 128 takes 308 and 328 us.
 static bool sweep_step(const StencilGeom& g, int64_t n, uint32_t nchunk, const float* Vc, const float* Vp, float* Vn,
                        const float* diag2, float o0, float o1, float o2, float c, float d, PanelOut po,
                        cudaStream_t s) {
     using ST = Tile3D;
     constexpr uint32_t C = SWEEP_C;
     if ((uint64_t)n * nchunk * 16 < (64ull << 20) || nchunk < (nchunk % C ? 24u : 12u)) return false;
+    const uint64_t plane = (uint64_t)g.d1 * g.d2;
+    const uint64_t tiled = (uint64_t)((g.d1 + ST::T1 - 1) / ST::T1) * ((g.d2 + ST::T2 - 1) / ST::T2) * ST::ROWS;
+    if (po.base && plane * nchunk * 16 < (8ull << 20) && 32 * tiled > 33 * plane) return false;
     const uint32_t ngrp = (nchunk + C - 1) / C;
     // about sixteen 256-thread CTAs an SM over the launch (its last wave is then a small
     // part), at least eight planes a run
