@@ -25,6 +25,8 @@ constexpr int KT = 32;  // rows per staged slab
 // the shape changes no bit of the result.  Float64 runs at 2 fma a clock and SM here: the
 // kernel is bound by the fma pipe (97 % busy), and what counts is that no warp multiplies
 // padding and that the chains are spread over the SMs.
+//   Broad: 64 x 64 tiles of eight 32 x 16 warp pieces, float32 only: there shared memory is
+//     the bound, and 16 outputs from 8 loads a lane take less of it than 8 from 6.
 //   Wide: 32 x 32 tiles of four 16 x 16 warp pieces.  Pieces past n_tot or below the
 //     diagonal idle.  The Gram pair of two 65536 x 200 float64 blocks: 8.05 ms, 13.7 ms
 //     with 64 x 64 tiles computed whole (1.77 times the useful products; 6.3 ms is the
@@ -38,6 +40,7 @@ constexpr int KT = 32;  // rows per staged slab
 // ST: staged slabs (more than two did not help the small tiles).  Staged with 16-byte
 // copies where rows are whole 16-byte units: 7.2 ms a call of the 32 x 32 grid, 40 probes,
 // degree 200, against 7.7 with 8-byte ones (both with two outputs a lane).
+struct BroadTile { static constexpr int P = 4, Q = 4, WR = 2, WC = 4, ST = 2; };
 struct WideTile { static constexpr int P = 2, Q = 4, WR = 2, WC = 2, ST = 2; };
 struct MidTile { static constexpr int P = 2, Q = 4, WR = 1, WC = 1, ST = 2; };
 struct SmallTile { static constexpr int P = 1, Q = 1, WR = 1, WC = 2, ST = 2; };
@@ -196,7 +199,7 @@ int64_t gram_ctas(int n_tot, bool odd, int n_split) {
     return (t * (t + 1) / 2 + (odd ? t * t : 0)) * n_split;
 }
 
-// The widest tile that still gives every SM a CTA (a chain of 512 rows or more per output
+// The widest float64 tile that still gives every SM a CTA (a chain of 512 rows or more per output
 // runs either way; with fewer CTAs than SMs the pipes of the others would idle).
 template <typename T, typename Acc>
 cudaError_t gram(const T* A, const T* B, int ld, int n_tot, int64_t n_rows, int n_split, double* part,
@@ -204,6 +207,15 @@ cudaError_t gram(const T* A, const T* B, int ld, int n_tot, int64_t n_rows, int 
     int64_t rps = (n_rows + n_split - 1) / n_split;
     rps = (rps + KT - 1) / KT * KT;
     const int sms = device_sms();
+    if constexpr (sizeof(T) == 4) {
+        // 64-wide tiles with three CTAs or more an SM and at most 1/7 wider padding (16384 rows
+        // of 700 columns, 20 steps: Gram 12.3 ms, 18.1 in 32-wide tiles; 4096 of 512 1.93 and
+        // 2.52; 65536 of 200 6.63 and 7.17; but 4096 of 257, 320 CTAs, 1.14 and 0.98, 16384 of
+        // 160, padded to 192, 1.28 and 1.17)
+        const int broad = (n_tot + 63) / 64 * 64, wide = (n_tot + 31) / 32 * 32;
+        if (gram_ctas<BroadTile>(n_tot, B != nullptr, n_split) >= 3 * sms && 7 * broad <= 8 * wide)
+            return gram_launch<T, Acc, BroadTile>(A, B, ld, n_tot, n_rows, n_split, rps, part, s);
+    }
     if (gram_ctas<WideTile>(n_tot, B != nullptr, n_split) >= sms)
         return gram_launch<T, Acc, WideTile>(A, B, ld, n_tot, n_rows, n_split, rps, part, s);
     if (gram_ctas<MidTile>(n_tot, B != nullptr, n_split) >= sms)
