@@ -72,6 +72,11 @@ constexpr int TMEM_COLS = 512;
 // KPM line of a 127 x 131 x 125 grid, degree 300: 79.0 ms a call, 46.7 ms with eight).
 // Panels hold ceil(n_tot / 8) groups, not a multiple of two, which takes a quarter off
 // their bytes there.
+// Wide blocks keep one panel a stage, and the kernel alone is slower on them than with 128
+// threads and a copy a part (65536 x 200: 38.5 us cold, 36.5 then), but the call is faster (400
+// steps 14.1 ms, 14.6 then): held to 64 registers (four CTAs' worth, whatever the sharing) it
+// leaves more of the SM to the recurrence CTAs beside it.  With 96 registers, which the compiler
+// takes if it may, it is as slow alone and the call takes 14.4 ms.
 constexpr int SMEM_BYTES = 4 * 2 * PART_BYTES + 1024;
 
 struct TcArgs {

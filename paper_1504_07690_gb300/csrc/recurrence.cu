@@ -117,18 +117,16 @@ struct RowInfo {
     uint32_t has;  // bit a: neighbour a present; bit 31: row exists
 };
 
-// Operands of one (row, 16-byte chunk) item of a stencil step: the centre
+// Operands of one (row, 16-byte chunk) item of a float32 stencil step: the centre
 // value, the neighbour sums per axis, V_{k-1} and the folded diagonal.
-template <typename T>
 struct ItemLoads {
-    typename Vec16<T>::type x, s[3], vp;
-    T dg;
+    float4 x, s[3], vp;
+    float dg;
     bool ok;
 };
 
-template <typename T, typename VT = typename Vec16<T>::type>
-__device__ __forceinline__ void load_item(ItemLoads<T>& L, const RowInfo& ri, uint32_t i, uint32_t cc,
-                                          uint32_t nchunk, const VT* vc, const VT* vp, const T* diag2, bool need_vp) {
+__device__ __forceinline__ void load_item(ItemLoads& L, const RowInfo& ri, uint32_t i, uint32_t cc, uint32_t nchunk,
+                                          const float4* vc, const float4* vp, const float* diag2, bool need_vp) {
     L.ok = (ri.has >> 31) != 0;
     if (!L.ok) return;
     const size_t base = (size_t)i * nchunk;
@@ -137,12 +135,12 @@ __device__ __forceinline__ void load_item(ItemLoads<T>& L, const RowInfo& ri, ui
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const bool lo = (ri.has >> (2 * a)) & 1u, hi = (ri.has >> (2 * a + 1)) & 1u;
-        VT sacc = vzero(T(0));
+        float4 sacc = vzero(0.f);
         if (lo) sacc = vadd(sacc, ldg_stream(vc + (size_t)ri.nb[2 * a] * nchunk + cc));
         if (hi) sacc = vadd(sacc, ldg_stream(vc + (size_t)ri.nb[2 * a + 1] * nchunk + cc));
         L.s[a] = sacc;
     }
-    L.vp = need_vp ? ldg_stream(vp + base + cc) : vzero(T(0));
+    L.vp = need_vp ? ldg_stream(vp + base + cc) : vzero(0.f);
 }
 
 // A CTA owns one 32-row panel at a time (grid-stride over panels): the first
@@ -151,19 +149,18 @@ __device__ __forceinline__ void load_item(ItemLoads<T>& L, const RowInfo& ri, ui
 // every lane is busy; with PANEL each item's split-bf16 hi and lo parts go
 // straight to their place in the panel (8-byte stores: no shared-memory stage
 // and no barrier per panel, so more of these CTAs fit next to a Gram CTA).
-template <typename T, bool PANEL>
+template <bool PANEL>
 __global__ void __launch_bounds__(256, 4)
-stencil_step_kernel(const T* __restrict__ Vc, const T* __restrict__ Vp, T* __restrict__ Vn,
-                    const T* __restrict__ diag2, StencilGeom g, T o0, T o1, T o2, T c, T d,
+stencil_step_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp, float* __restrict__ Vn,
+                    const float* __restrict__ diag2, StencilGeom g, float o0, float o1, float o2, float c, float d,
                     uint32_t nchunk, uint32_t n_rows, PanelOut po) {
-    using VT = typename Vec16<T>::type;
     __shared__ RowInfo info[32];
     const uint32_t mdiv = ((1u << 20) + nchunk - 1) / nchunk;  // it / nchunk for it < 32 nchunk
-    const VT* vc = reinterpret_cast<const VT*>(Vc);
-    const VT* vp = reinterpret_cast<const VT*>(Vp);
-    VT* vn = reinterpret_cast<VT*>(Vn);
+    const float4* vc = reinterpret_cast<const float4*>(Vc);
+    const float4* vp = reinterpret_cast<const float4*>(Vp);
+    float4* vn = reinterpret_cast<float4*>(Vn);
     const uint32_t s1 = g.d2, s0 = g.d1 * g.d2;
-    const T w[3] = {g.active[0] ? o0 : T(0), g.active[1] ? o1 : T(0), g.active[2] ? o2 : T(0)};
+    const float w[3] = {g.active[0] ? o0 : 0.f, g.active[1] ? o1 : 0.f, g.active[2] ? o2 : 0.f};
     const uint32_t n_pan = (n_rows + 31) / 32;
     const uint32_t items = 32 * nchunk;
     for (uint32_t pnl = blockIdx.x; pnl < n_pan; pnl += gridDim.x) {
@@ -191,7 +188,7 @@ stencil_step_kernel(const T* __restrict__ Vc, const T* __restrict__ Vp, T* __res
         __syncthreads();
         // two items per thread per pass, all their loads issued before either is used
         for (uint32_t it0 = threadIdx.x; it0 < items; it0 += 2 * blockDim.x) {
-            ItemLoads<T> L[2];
+            ItemLoads L[2];
             uint32_t rr[2], cq[2];
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
@@ -202,20 +199,20 @@ stencil_step_kernel(const T* __restrict__ Vc, const T* __restrict__ Vp, T* __res
                 if (it < items) {
                     rr[u] = (it * mdiv) >> 20;
                     cq[u] = it - rr[u] * nchunk;
-                    load_item(L[u], info[rr[u]], pnl * 32 + rr[u], cq[u], nchunk, vc, vp, diag2, d != T(0));
+                    load_item(L[u], info[rr[u]], pnl * 32 + rr[u], cq[u], nchunk, vc, vp, diag2, d != 0.f);
                 }
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const uint32_t it = it0 + u * blockDim.x;
                 if (it >= items) continue;
-                VT out = vzero(T(0));
+                float4 out = vzero(0.f);
                 if (L[u].ok) {
-                    VT acc = vscale(L[u].dg, L[u].x);
+                    float4 acc = vscale(L[u].dg, L[u].x);
 #pragma unroll
                     for (int a = 0; a < 3; ++a) acc = vfma(w[a], L[u].s[a], acc);
                     out = vscale(c, acc);
-                    if (d != T(0)) out = vfma(-d, L[u].vp, out);
+                    if (d != 0.f) out = vfma(-d, L[u].vp, out);
                     vn[(size_t)(pnl * 32 + rr[u]) * nchunk + cq[u]] = out;
                 }
                 if constexpr (PANEL) panel_store4(po, pnl, rr[u], 4 * cq[u], out);
@@ -381,7 +378,7 @@ stencil_march_kernel(const float* __restrict__ Vc, const float* __restrict__ Vp,
 // ms a call against 61.6 ms on the 256^2 one.)  Four CTAs an SM, 64 registers a thread: with
 // the 79 that the compiler takes for fewer a call on the 64^3 grid takes 71.3 ms instead of 63.7
 // (256 columns, 128 of them hybrid, degree 300, 400 pencils).
-using Tile3D = SweepTile<8, 8, 1>;
+using Tile3D = SweepTile<8, 8>;
 constexpr uint32_t SWEEP_C = 4;
 
 template <bool PANEL>
@@ -633,7 +630,7 @@ static cudaError_t stencil_step_f32(const Plan& P, const float* Vc, const float*
         }
         if (sweep_step(P.geom, P.n, nchunk, Vc, Vp, Vn, diag2, o0, o1, o2, c, d, po, s)) return cudaGetLastError();
     }
-    const auto kernel = panel ? stencil_step_kernel<float, true> : stencil_step_kernel<float, false>;
+    const auto kernel = panel ? stencil_step_kernel<true> : stencil_step_kernel<false>;
     kernel<<<panel_grid(P.n), stencil_threads(nchunk), 0, s>>>(Vc, Vp ? Vp : Vc, Vn, diag2, P.geom, o0, o1, o2, c, d,
                                                                nchunk, (uint32_t)P.n, po);
     return cudaGetLastError();

@@ -1,16 +1,18 @@
 // sweep.cuh - shared pieces of the kernels that sweep the planes of a grid along axis 0
 // (stencil steps in recurrence.cu, the adjoint step in adjoint.cu).
 //
-// A CTA owns a T1 x T2 tile of axes 1 and 2 and a run of planes.  The tile's planes (with
-// their halo) go through a ring of shared-memory slots filled by asynchronous copies, PF
-// planes ahead, so that the loads in flight take no registers.
+// A CTA owns a T1 x T2 tile of axes 1 and 2 and a run of planes.  The adjoint step's planes
+// (with their halo) go through a ring of shared-memory slots filled by asynchronous copies,
+// PF planes ahead, so that the loads in flight take no registers.  The forward step keeps
+// three planes of its element in registers and only the current one, with its halo, in
+// shared memory (PF = 0: no ring).
 #pragma once
 
 #include "internal.h"
 
 namespace ssm {
 
-template <int T1_, int T2_, int PF_>
+template <int T1_, int T2_, int PF_ = 0>
 struct SweepTile {
     static constexpr int T1 = T1_, T2 = T2_, ROWS = T1 * T2, W2 = T2 + 2;
     static constexpr int H1 = T1 > 1 ? 1 : 0;             // halo along axis 1 (T1 = 1: the axis is inactive)
