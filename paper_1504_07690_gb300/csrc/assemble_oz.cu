@@ -228,9 +228,9 @@ template <int NS>
 __global__ void __launch_bounds__(NTHREADS, 1) assemble_oz_kernel(AsmArgs P) {
     constexpr int A_STAGE = a_stage<NS>(), B_STAGE = b_stage<NS>();
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ uint64_t full[SST], empty[SST], a_full, a_empty;
+    __shared__ uint64_t full[SST], empty[SST], a_full, a_empty, drained;
     __shared__ uint32_t tmem_slot;
-    __shared__ int fail;
+    __shared__ int fail, issued;  // issued: stages copied
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tt = blockIdx.x, et = blockIdx.y;  // the point tiles of an entry tile run together:
                                                  // its moment slices come from L2 after the first
@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) assemble_oz_kernel(AsmArgs P) {
         }
         mbar_init(&a_full, 1);
         mbar_init(&a_empty, NDRAIN);
+        mbar_init(&drained, 1);
         fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
@@ -258,7 +259,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) assemble_oz_kernel(AsmArgs P) {
 
     if (warp == 0) {
         if (lane == 0) {  // producer
-            for (int q = 0; q < nst; ++q) {
+            int q = 0;
+            for (; q < nst; ++q) {
                 const int s = q % SST;
                 if (q >= SST && !mbar_spin(smem_u32(&empty[s]), ((q / SST) - 1) & 1, &fail)) {
                     atomicOr(&fail, 1);
@@ -269,6 +271,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) assemble_oz_kernel(AsmArgs P) {
                 bulk_copy(dst, xsrc + (size_t)q * A_STAGE, (uint32_t)A_STAGE, &full[s]);
                 bulk_copy(dst + A_STAGE, csrc + (size_t)q * B_STAGE, (uint32_t)B_STAGE, &full[s]);
             }
+            issued = q;
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -370,7 +373,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) assemble_oz_kernel(AsmArgs P) {
         }
     }
     __syncthreads();
-    if (fail && tid == 0) atomicOr(P.flag, 2);
+    if (fail) {  // shared memory and TMEM are not given up under copies and MMAs on their way
+        if (tid == 0) {
+            atomicOr(P.flag, 2);
+            wait_copies(full, SST, 0, issued);
+        }
+        if (tid == 32) {
+            umma_commit(&drained);
+            mbar_wait_sleep(smem_u32(&drained), 0, nullptr);
+        }
+        __syncthreads();
+    }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0) tmem_dealloc(tmem, 512);
 }

@@ -46,8 +46,8 @@
 // suspended on the mbarrier (try_wait with a time hint) rather than polling,
 // so they leave the issue slots to the working warps.  Every wait is bounded
 // and also ends when another thread has recorded a failure; on failure the
-// CTA sets bit 2 of the status word, waits (bounded) for its MMAs, frees
-// TMEM and returns.
+// CTA sets bit 2 of the status word, waits (bounded) for its MMAs and copies,
+// frees TMEM and returns.
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fused_step_tc_kernel(FArgs P) {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t xfull[MAX_X], xempty[MAX_X], full[MAX_S], empty[MAX_S], done;
     __shared__ uint32_t tmem_slot;
-    __shared__ int fail;
+    __shared__ int fail, copied;  // copied: panels the loader issued
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool t1 = (int)blockIdx.x >= P.a_ctas;
     const int64_t first = t1 ? (int64_t)blockIdx.x - P.a_ctas : (int64_t)blockIdx.x;
@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(FTHREADS, 1) fused_step_tc_kernel(FArgs P) {
         const uint32_t s1 = P.g.d2, s0 = P.g.d1 * P.g.d2;
         const char* xsrc = reinterpret_cast<const char*>(t1 ? P.Xb : P.Vc);
         const char* ysrc = reinterpret_cast<const char*>(t1 ? P.Yb : P.Vp);
-        for (int c = 0; c < nch; ++c) {
+        int c = 0;
+        for (; c < nch; ++c) {
             const int sx = c % NX;
             bool okw = c < NX || mbar_wait_sleep(smem_u32(&xempty[sx]), ((c / NX) - 1) & 1, vfail);
             okw = __all_sync(0xffffffffu, okw);  // one decision for the whole warp
@@ -315,6 +316,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fused_step_tc_kernel(FArgs P) {
             }
             if (lane != 0) mbar_arrive(bar);  // lane 0 arrived with the byte count
         }
+        if (lane == 0) copied = c;
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
         if (lane == 0) {
@@ -514,6 +516,7 @@ __global__ void __launch_bounds__(FTHREADS, 1) fused_step_tc_kernel(FArgs P) {
         }
     } else if (!ok && tid == 0) {
         atomicOr(P.flag, 2);
+        wait_copies(xfull, NX, 0, copied);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

@@ -44,7 +44,8 @@
 // kind::f16 into TMEM, and eight of the converting warps drain the
 // accumulators at the start of each interval.  The hand-offs spin on the
 // mbarriers (mbarrier.test_wait).  Every wait is bounded; on expiry the CTA
-// sets bit 2 of the status word and stops.
+// sets bit 2 of the status word, waits once more (bounded) for its copies and MMAs, frees
+// TMEM and stops.
 //
 // What bounds it: instruction issue in the converting warps and the one-thread MMA loop,
 // not the tensor pipe.  Two values an instruction in the splitting (f32x2), one multiply
@@ -159,9 +160,9 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
 
 __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ uint64_t f_full[FST], f_empty[FST], s_full[SST], s_empty[SST], a_full, a_empty;
+    __shared__ uint64_t f_full[FST], f_empty[FST], s_full[SST], s_empty[SST], a_full, a_empty, drained;
     __shared__ uint32_t tmem_slot;
-    __shared__ int fail;
+    __shared__ int fail, issued;  // issued: stages copied
     __shared__ __align__(16) float escale[MAXN];  // 2^-E of each column
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
         }
         mbar_init(&a_full, 1);
         mbar_init(&a_empty, NEPI);
+        mbar_init(&drained, 1);
         fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
@@ -249,7 +251,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
     if (warp == 0) {
         if (lane == 0) {  // producer: float-pair rows into the staging ring
             const uint32_t rb = (uint32_t)(T.ncopy * 4);
-            for (int q = 0; q < nst; ++q) {
+            int q = 0;
+            for (; q < nst; ++q) {
                 const int fs = q % nf;
                 if (q >= nf && !mbar_spin(smem_u32(&f_empty[fs]), ((q / nf) - 1) & 1, &fail)) {
                     atomicOr(&fail, 1);
@@ -263,6 +266,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
                 bulk_copy(dst, Yh + src, (uint32_t)nr * rb, &f_full[fs]);
                 bulk_copy(dst + (uint32_t)(KS * fpitch), Yl + src, (uint32_t)nr * rb, &f_full[fs]);
             }
+            issued = q;
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -468,9 +472,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_oz_kernel(OzArgs P) {
         if (epi && alive && niv > 0) drain(niv - 1);
     }
     // teardown: every issued MMA has completed before TMEM is released (the last
-    // commit on a_full covers all of them, and the epilogue waited for it)
+    // commit on a_full covers all of them, and the epilogue waited for it; after a failure
+    // the issuer waits for them here)
     __syncthreads();
-    if (fail && tid == 0) atomicOr(P.flag, 2);
+    if (fail) {
+        if (tid == 0) {
+            atomicOr(P.flag, 2);
+            wait_copies(f_full, nf, 0, issued);
+        }
+        if (tid == 32) {
+            umma_commit(&drained);
+            mbar_wait_sleep(smem_u32(&drained), 0, nullptr);
+        }
+        __syncthreads();
+    }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 0) tmem_dealloc(tmem, 512);
 }

@@ -35,7 +35,7 @@
 // shared-memory footprint keeps it alone on its SM (two or four CTAs with their parts of
 // each share an SM where slabs are small and blocks narrow).  Every wait is bounded:
 // on expiry the CTA sets bit 2 of the status word, waits once more (bounded)
-// for its MMAs, frees TMEM and returns.
+// for its copies and MMAs, frees TMEM and returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) gram_tc_kernel(TcArgs P) {
                 const int s = c % nstage;
                 if (!mbar_wait_sleep(smem_u32(&full[s]), (c / nstage) & 1, nullptr)) {
                     ok = false;
+                    wait_copies(full, nstage, c, min(nsg, c + nstage));  // those before have landed
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) gram_tc_kernel(TcArgs P) {
                 umma_commit(&empty[s]);
             }
             if (!ok) atomicOr(&fail, 1);
-            if (nch > 0 && ok)
+            if (acc)
                 umma_commit(&done);  // arrives once every MMA issued above has completed
             else
                 mbar_arrive(&done);

@@ -147,6 +147,14 @@ __device__ __forceinline__ void umma_commit(uint64_t* m) {
                  : "memory");
 }
 
+// Bounded wait, after a failure, for copies c0 .. c1 - 1 of those issued in order into a ring of
+// nb barriers (at most the last nb): shared memory must not be given up with a copy on its
+// way into it.  Ends at the first that does not land.
+__device__ __forceinline__ void wait_copies(uint64_t* full, int nb, int c0, int c1) {
+    for (int c = c0 > c1 - nb ? c0 : c1 - nb; c < c1; ++c)
+        if (!mbar_wait_sleep(smem_u32(&full[c % nb]), (c / nb) & 1, nullptr)) return;
+}
+
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
                  "r"(cols));
